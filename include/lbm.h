@@ -353,7 +353,8 @@ lbm_status lbm_batch_set_f(lbm_ctx *ctx, int case_index, const float *f);
 
 /* lbm_step(ctx, n) with n >= 4 on a non-default stream replays two steps
    captured once into a CUDA graph (the first such call also runs two plain
-   steps before capturing).  enable = 0 launches every step directly.  The
+   steps before capturing); 16 steps, from n >= 20, in the box form of small
+   lattices.  enable = 0 launches every step directly.  The
    result does not depend on it. */
 lbm_status lbm_set_graphs(lbm_ctx *ctx, int enable);
 

@@ -95,6 +95,8 @@ def tune(ctx, params_list, stream, steps=8, cache_path=DEFAULT_CACHE, use_cache=
         shapes = BATCH_SHAPES if len(params_list) > 1 else SINGLE_SHAPES
         nz = max(p.nz for p in params_list)
         candidates = [(ty, zc, hold) for ty, hold in shapes for zc in ZCHUNKS if zc <= max(nz, 8)]
+        if len(params_list) == 1:  # the context's own choice (small lattices: the box form)
+            candidates.insert(0, lbm.lbm_get_fused_config(ctx))
     best = None
     for ty, zc, hold in candidates:
         try:

@@ -28,6 +28,9 @@ struct lbm_ctx {
   int ncases;
   int storage, kernel;
   lbm::FusedConfig fused;
+  lbm::FusedConfig fused_default;  // the configuration create picked
+  int box_default;                 // ... and its box form (0: none), single lattices
+  int box;                         // box form in use: box_default while `fused` is the default
   cudaStream_t stream;
   int device, sms;
   size_t elem;              // bytes per stored population value
@@ -70,11 +73,14 @@ struct lbm_ctx {
   int total_items;
   int plate_axis;           // axis of the moving plates (wall = 2), or -1
   double plate_u[2][3];     // their velocities (low, high)
-  cudaGraphExec_t graph;    // two captured steps (buffer 0 -> 1 -> 0)
+  cudaGraphExec_t graph;    // captured steps (buffer 0 -> 1 -> ... -> 0)
+  int graph_steps;          // their number, even
   int use_graph;
   long long steps;
   char err[512];
 };
+
+constexpr int kBoxGraphSteps = 16;
 
 static thread_local char g_create_err[512];
 
@@ -577,6 +583,8 @@ static lbm_status create_ctx(const lbm_params* ps, int ncases, void* cuda_stream
       }
     }
   }
+  if (st == LBM_OK && ncases == 1 && c->kernel == LBM_KERNEL_FUSED)
+    c->box_default = c->box = lbm::default_box(c->cases[0].args, c->storage);
   if (st == LBM_OK && ncases > 1) {
     // tensor maps of every case for the batched TMA step (tile kinds 0, 2)
     bool all = true;
@@ -638,6 +646,7 @@ static lbm_status create_ctx(const lbm_params* ps, int ncases, void* cuda_stream
   if (st == LBM_OK && ncases > 1 &&
       lbm::dev_alloc((void**)&c->d_cases, sizeof(lbm::BatchCase) * ncases) != cudaSuccess)
     st = fail(nullptr, LBM_ERR_OOM, "cudaMalloc of the case table failed");
+  c->fused_default = c->fused;
   if (st == LBM_OK) {
     st = upload_case_table(c);
     if (st != LBM_OK) {
@@ -835,6 +844,8 @@ static lbm_status launch_step(lbm_ctx* c, int from, lbm::MonAcc* mon = nullptr) 
     e = lbm::launch_fused_batch(c->storage, src, dst, c->d_cases, c->ncases,
                                 c->total_items, c->any_walls, c->cases[0].args.bgk != 0,
                                 c->fused, c->sms, c->stream);
+  else if (c->box && !mon)
+    e = lbm::launch_fused_box(c->storage, src, dst, c->cases[0].args, c->box, c->stream);
   else if (c->kernel == LBM_KERNEL_TWO_PASS)
     e = lbm::launch_twopass(c->storage, src, dst, c->cases[0].args, c->phase, c->stream);
   else if (c->seam16_ok && c->fused.hold == 7 &&
@@ -866,14 +877,17 @@ static lbm_status launch_step(lbm_ctx* c, int from, lbm::MonAcc* mon = nullptr) 
   return LBM_OK;
 }
 
-// Two steps (buffer 0 -> 1 -> 0) captured once into a CUDA graph.
+// Steps (buffer 0 -> 1 -> ... -> 0) captured once into a CUDA graph: two, or
+// kBoxGraphSteps of the box form, whose steps are shorter than the gap
+// between two graph launches.
 static lbm_status ensure_graph(lbm_ctx* c) {
   if (c->graph) return LBM_OK;
+  c->graph_steps = c->box ? kBoxGraphSteps : 2;
   cudaGraph_t g = nullptr;
   LBM_CUDA(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal),
            "cudaStreamBeginCapture");
-  lbm_status st = launch_step(c, 0);
-  if (st == LBM_OK) st = launch_step(c, 1);
+  lbm_status st = LBM_OK;
+  for (int k = 0; k < c->graph_steps && st == LBM_OK; ++k) st = launch_step(c, k & 1);
   cudaError_t e = cudaStreamEndCapture(c->stream, &g);
   if (st != LBM_OK) {
     if (g) cudaGraphDestroy(g);
@@ -901,7 +915,7 @@ extern "C" lbm_status lbm_step(lbm_ctx* c, int n) {
     if (sd != LBM_OK) return sd;
   }
   // CUDA graphs need a capturable stream (not the legacy default stream).
-  const bool graphs = c->use_graph && c->stream != nullptr && n >= 4;
+  const bool graphs = c->use_graph && c->stream != nullptr && n >= (c->box ? kBoxGraphSteps + 4 : 4);
   lbm_status st;
   if (graphs) {
     // Bring the state to buffer 0; before the first capture also run two
@@ -915,9 +929,9 @@ extern "C" lbm_status lbm_step(lbm_ctx* c, int n) {
       n -= 1;
     }
     if ((st = ensure_graph(c)) != LBM_OK) return st;
-    for (; n >= 2; n -= 2) {
+    for (; n >= c->graph_steps; n -= c->graph_steps) {
       LBM_CUDA(c, cudaGraphLaunch(c->graph, c->stream), "cudaGraphLaunch");
-      c->steps += 2;
+      c->steps += c->graph_steps;
     }
   }
   for (; n > 0; --n) {
@@ -1286,6 +1300,15 @@ extern "C" lbm_status lbm_set_planes(lbm_ctx* c, int z0, int n, const void* src)
   return plane_copy(c, z0, n, const_cast<void*>(src), false);
 }
 
+// A configuration set explicitly runs the marching kernel it names; the one
+// that create picked brings back create's choice, the box form included.
+static void use_config(lbm_ctx* c, const lbm::FusedConfig& f) {
+  const lbm::FusedConfig& d = c->fused_default;
+  c->fused = f;
+  c->box = f.tile_y == d.tile_y && f.zchunk == d.zchunk && f.hold == d.hold ? c->box_default : 0;
+  drop_graph(c);
+}
+
 extern "C" lbm_status lbm_set_fused_config(lbm_ctx* c, int tile_y, int zchunk,
                                            int hold) {
   if (!c) return LBM_ERR_ARG;
@@ -1313,8 +1336,7 @@ extern "C" lbm_status lbm_set_fused_config(lbm_ctx* c, int tile_y, int zchunk,
         return fail(c, LBM_ERR_ARG,
                     "tile_y 12 is the batched seam form (hold 7) of FP32 batches whose cases "
                     "are periodic in x and y (MRT, nx a multiple of 2)");
-      c->fused = f;
-      drop_graph(c);
+      use_config(c, f);
       lbm_status st = upload_case_table(c);
       if (st != LBM_OK) return st;
       c->err[0] = 0;
@@ -1325,8 +1347,7 @@ extern "C" lbm_status lbm_set_fused_config(lbm_ctx* c, int tile_y, int zchunk,
                   "tile_y 12 is the two-stage seam form (hold 7) of single periodic lattices "
                   "with nx a multiple of 2 (FP32) or 4 (16-bit), nx >= 34 and ny >= 15");
     if (zchunk == 0) f.zchunk = lbm::seam12_zchunk(c->cases[0].args, c->sms);
-    c->fused = f;
-    drop_graph(c);
+    use_config(c, f);
     c->err[0] = 0;
     return LBM_OK;
   }
@@ -1342,8 +1363,7 @@ extern "C" lbm_status lbm_set_fused_config(lbm_ctx* c, int tile_y, int zchunk,
                       "0..8; hold 2, 3, 5, 6 need tile_y 8, hold 4 needs tile_y 16, tile_y 15 "
                       "needs hold 7 or 8; hold 7 and 8 need nx * pair bytes a multiple of 16 "
                       "and a tile whose stages fit shared memory)");
-  c->fused = f;
-  drop_graph(c);
+  use_config(c, f);
   lbm_status st = upload_case_table(c);
   if (st != LBM_OK) return st;
   c->err[0] = 0;

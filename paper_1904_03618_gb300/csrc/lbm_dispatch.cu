@@ -18,6 +18,16 @@ cudaError_t launch_fused(int storage, const void* src, void* dst,
   return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_fused_box(int storage, const void* src, void* dst, const StepArgs& a, int box,
+                             cudaStream_t s) {
+  switch (storage) {
+    case 0: return launch_fused_box_storage<float>(src, dst, a, box, s);
+    case 1: return launch_fused_box_storage<__half>(src, dst, a, box, s);
+    case 2: return launch_fused_box_storage<__nv_bfloat16>(src, dst, a, box, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
 cudaError_t launch_fused_batch(int storage, const void* src, void* dst,
                                const BatchCase* cases, int ncases,
                                int total_items, bool walls, bool bgk,
@@ -328,6 +338,20 @@ FusedConfig default_fused_config(const StepArgs& a, int storage) {
   if (zc > a.nz) zc = a.nz;
   c.zchunk = zc;
   return c;
+}
+
+// The box form's range, GB300, us per step (box / marching kernel): it wins
+// up to about 260,000 cells (FP32 56^3 16.3 / 25.0, 64^3 24.2 / 27.6, 80^3
+// 48 / 43; FP16 64^3 21.5 / 28.7; 65 x 64 x 64 with walls 35 / 36).  On the
+// lattices of the seam forms, the line lies lower than that, at 81,920
+// cells: from there on the tensor-copy kernel with its bounded waits, which
+// reports them in the error word, is the documented default (the fault tests
+// step a 64 x 40 x 36 lattice through it).
+int default_box(const StepArgs& a, int storage) {
+  const long long N = (long long)a.nx * a.ny * a.nz;
+  const bool seam = seam_eligible(a, storage) || seam16_eligible(a, storage);
+  if (N > (seam ? 81920 : 262144)) return 0;
+  return N <= 16384 ? 1 : 2;
 }
 
 }  // namespace lbm

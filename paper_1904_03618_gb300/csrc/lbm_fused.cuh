@@ -162,16 +162,14 @@ __device__ __forceinline__ void store_recoloured(T* dst, unsigned plane,
   StoreRecoloured<T, 1>::run(dst, plane, a, c, rc, fs);
 }
 
-// Eq. 49 gradients of rho^N and the correction fluxes at an interior cell
-// from the shared window, as weighted differences of opposite neighbours so
-// that a uniform field gives an exactly zero gradient.  A neighbour beyond a
-// wall takes the centre value.
-template <int BY, int TW = kTileW>
-__device__ __forceinline__ void window_gradients(
-    const float4 (*win)[BY][TW], int z, int ty, int tx, bool xlo, bool xhi,
-    bool ylo, bool yhi, bool zlo, bool zhi, float4& ctr, float& Gx, float& Gy,
-    float& Gz, float& Qx, float& Qy, float& Qz) {
-  ctr = win[z & 3][ty][tx];
+// Eq. 49 gradients of rho^N and the correction fluxes at an interior cell,
+// as weighted differences of opposite neighbours so that a uniform field
+// gives an exactly zero gradient.  at(dx, dy, dz) is the window entry of a
+// neighbour; one beyond a wall takes the centre value ctr.
+template <typename At>
+__device__ __forceinline__ void stencil_gradients(
+    const At& at, const float4& ctr, bool xlo, bool xhi, bool ylo, bool yhi, bool zlo, bool zhi,
+    float& Gx, float& Gy, float& Gz, float& Qx, float& Qy, float& Qz) {
   Gx = Gy = Gz = Qx = Qy = Qz = 0.f;
 #pragma unroll
   for (int i = 1; i < 19; i += 2) {
@@ -180,8 +178,8 @@ __device__ __forceinline__ void window_gradients(
                     (dy < 0 && ylo) || (dz > 0 && zhi) || (dz < 0 && zlo);
     const bool bm = (dx < 0 && xhi) || (dx > 0 && xlo) || (dy < 0 && yhi) ||
                     (dy > 0 && ylo) || (dz < 0 && zhi) || (dz > 0 && zlo);
-    const float4 vp = bp ? ctr : win[(z + dz) & 3][ty + dy][tx + dx];
-    const float4 vm = bm ? ctr : win[(z - dz) & 3][ty - dy][tx - dx];
+    const float4 vp = bp ? ctr : at(dx, dy, dz);
+    const float4 vm = bm ? ctr : at(-dx, -dy, -dz);
     const float w = (i <= 6) ? (1.0f / 6.0f) : (1.0f / 12.0f);
     if (dx) {
       Gx += (dx * w) * (vp.x - vm.x);
@@ -196,6 +194,19 @@ __device__ __forceinline__ void window_gradients(
       Qz += (dz * w) * (vp.w - vm.w);
     }
   }
+}
+// The same from the marching kernels' four-slot window (plane index mod 4).
+template <int BY, int TW = kTileW>
+__device__ __forceinline__ void window_gradients(
+    const float4 (*win)[BY][TW], int z, int ty, int tx, bool xlo, bool xhi,
+    bool ylo, bool yhi, bool zlo, bool zhi, float4& ctr, float& Gx, float& Gy,
+    float& Gz, float& Qx, float& Qy, float& Qz) {
+  ctr = win[z & 3][ty][tx];
+  stencil_gradients(
+      [&](int dx, int dy, int dz) -> const float4& {
+        return win[(z + dz) & 3][ty + dy][tx + dx];
+      },
+      ctr, xlo, xhi, ylo, yhi, zlo, zhi, Gx, Gy, Gz, Qx, Qy, Qz);
 }
 
 // Per-thread geometry shared by the kernels: a CTA tile of TW x BY columns

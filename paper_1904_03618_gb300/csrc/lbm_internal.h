@@ -112,6 +112,15 @@ cudaError_t launch_fused(int storage, const void* src, void* dst,
                          const StepArgs& a, const FusedConfig& cfg,
                          cudaStream_t s);
 FusedConfig default_fused_config(const StepArgs& a, int storage);
+// Box form of the step for small lattices (lbm_fused_box.cuh): box 1 = 4 x 4
+// x 4 cells per CTA, 2 = 8 x 4 x 4; default_box 0: the lattice is large
+// enough for the marching kernels.
+int default_box(const StepArgs& a, int storage);
+template <typename T>
+cudaError_t launch_fused_box_storage(const void* src, void* dst, const StepArgs& a, int box,
+                                     cudaStream_t s);
+cudaError_t launch_fused_box(int storage, const void* src, void* dst, const StepArgs& a, int box,
+                             cudaStream_t s);
 
 // TMA-staged fused step (hold 7: two stages, hold 8: one stage).  Tile
 // kinds: 0 = 32 x 8 threads (tile_y 8), 1 = 16 x 16 (tile_y 16), 2 = 34 x 15
