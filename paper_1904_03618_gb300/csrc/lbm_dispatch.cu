@@ -199,6 +199,11 @@ cudaError_t tma_build_maps(int storage, const void* base, const StepArgs& a, int
   return cudaSuccess;
 }
 
+// z chunk in [lo, hi] whose list schedule of cols x ceil(nz / chunk) CTAs over
+// `slots` places ends first, a CTA of p planes costing p + overhead (ties: the
+// longer chunk); at most nz.
+static int schedule_zchunk(long long cols, int nz, int slots, int lo, int hi, double overhead);
+
 int seam12_zchunk(const StepArgs& a, int sms) { return list_schedule_zchunk(a, sms, 10); }
 
 int list_schedule_zchunk(const StepArgs& a, int sms, int rows) {
@@ -216,16 +221,18 @@ int list_schedule_zchunk(const StepArgs& a, int sms, int rows) {
   // FP32 and 1.6-3.2 % slower at 160^3; beyond 48 planes the CTAs marching
   // neighbouring columns drift apart and the model, which does not see
   // that, goes wrong (128 planes on the 1024-plane lattice: 12 % slower).
-  constexpr double kOverhead = 3.0;
   const long long cols = (long long)((a.nx + 31) / 32) * ((a.ny + rows - 1) / rows);
-  const int slots = sms > 0 ? sms : 152;
+  return schedule_zchunk(cols, a.nz, sms > 0 ? sms : 152, 6, 48, 3.0);
+}
+
+static int schedule_zchunk(long long cols, int nz, int slots, int lo, int hi, double overhead) {
   std::vector<double> heap((size_t)slots);
   int best_zc = 12;
   double best_span = 1e300;
-  for (int zc = 6; zc <= 48; ++zc) {
-    const long long full = (long long)(a.nz / zc) * cols;
-    const int tail = a.nz % zc;
-    const double d = zc + kOverhead;
+  for (int zc = lo; zc <= hi; ++zc) {
+    const long long full = (long long)(nz / zc) * cols;
+    const int tail = nz % zc;
+    const double d = zc + overhead;
     const long long rounds = full / slots, extra = full % slots;
     for (int j = 0; j < slots; ++j) heap[(size_t)j] = (double)(rounds + (j < extra)) * d;
     double span = (double)(rounds + (extra > 0)) * d;
@@ -234,7 +241,7 @@ int list_schedule_zchunk(const StepArgs& a, int sms, int rows) {
       std::make_heap(heap.begin(), heap.end(), later);
       for (long long c = 0; c < cols; ++c) {
         std::pop_heap(heap.begin(), heap.end(), later);
-        heap.back() += tail + kOverhead;
+        heap.back() += tail + overhead;
         span = std::max(span, heap.back());
         std::push_heap(heap.begin(), heap.end(), later);
       }
@@ -244,7 +251,7 @@ int list_schedule_zchunk(const StepArgs& a, int sms, int rows) {
       best_zc = zc;
     }
   }
-  return best_zc < a.nz ? best_zc : a.nz;
+  return best_zc < nz ? best_zc : nz;
 }
 
 bool seam_eligible(const StepArgs& a, int storage) {
@@ -321,22 +328,22 @@ bool valid_fused_config(const FusedConfig& c, int storage) {
   return c.zchunk > 0;
 }
 
-// Default: 30 x 6 interior tiles, reduced state held in shared memory, and
-// chunks of 12 planes (each chunk re-reads two extra planes for its halo),
-// shortened down to 4 planes while the grid has fewer than two CTAs per SM
-// over the 152 SMs.  Measured on GB300 at 128^3 (FP32 and FP16 storage):
-// 8- and 12-plane chunks are best; 16, 24 and 32 are slower, as are the
-// register-capped, two-rows-per-thread and cp.async-pipelined variants.
+// Default: 30 x 6 interior tiles, reduced state held in shared memory, two
+// CTAs per SM.  The z chunk is the one whose list schedule over the 2 x 152
+// slots ends first, as for the seam forms (list_schedule_zchunk); halo planes
+// and start cost 2.5 planes here.  GB300, us per step, against 12 planes halved
+// while the grid left slots empty: 101 x 99 x 67 with walls 16 planes 61.7, 12
+// planes 81.5 (408 CTAs for 304 slots: a second round a third full); 129 x 65
+// x 150 28 planes 108, 12 planes 122; 200 x 100 x 100 BGK 41 planes 149, 12
+// planes 161; within 4 % of the fastest of 15 chunks on seven odd, walled and
+// 16-bit lattices.
 FusedConfig default_fused_config(const StepArgs& a, int storage) {
   (void)storage;
   FusedConfig c;
   c.tile_y = 8;
   c.hold = 2;
   const long long cols = (long long)((a.nx + 29) / 30) * ((a.ny + 5) / 6);
-  int zc = 12;
-  while (zc > 4 && cols * ((a.nz + zc - 1) / zc) < 2 * 152) zc /= 2;
-  if (zc > a.nz) zc = a.nz;
-  c.zchunk = zc;
+  c.zchunk = schedule_zchunk(cols, a.nz, 2 * 152, 3, 48, 2.5);
   return c;
 }
 
