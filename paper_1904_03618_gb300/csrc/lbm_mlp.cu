@@ -3,9 +3,11 @@
 // The network maps impact parameters to a spreading-factor series: dense
 // layers x -> tanh(x W + b) -> ... -> (. W_out + b_out), trained with mean
 // squared error and Adam.  Every matrix product of the forward and backward
-// passes runs on the tensor cores, in k_gemm_ws when its K is at most 256
-// (every forward layer and dZ W^T; a persistent warp-specialised kernel,
-// described above it) and otherwise in k_gemm_tc:
+// passes runs on the tensor cores: inference and training steps of up to 4096
+// rows in the whole-network kernels of lbm_net.cuh; the products of larger
+// training batches (and lbm_gemm_bf16) in k_gemm_ws when K is at most 256
+// (a persistent warp-specialised kernel, described above it) or split over
+// it, and otherwise in k_gemm_tc:
 //   - a CTA owns a 128-row tile of C (all of C's columns, N <= 256);
 //   - the A (128 x 64) and B (N x 64) K-slices are converted to BF16 and
 //     written into shared memory in the canonical K-major layout without
@@ -1328,22 +1330,12 @@ __global__ void k_colsum(const float* __restrict__ dz, int rows, int cols,
   db[n] = s;
 }
 
-// One Adam step over all parameters (bias-corrected, Kingma & Ba).
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g,
-                       float* __restrict__ m, float* __restrict__ v, long long n, float lr,
-                       float b1, float b2, float eps, float c1, float c2) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-}
-
 }  // namespace mlp
+}  // namespace lbm
 
+#include "lbm_net.cuh"
+
+namespace lbm {
 cudaError_t mlp_set_wait_ns(unsigned long long ns) {
   const unsigned long long v = ns ? ns : mlp::kWaitNs;
   return cudaMemcpyToSymbol(mlp::g_mma_wait_ns, &v, sizeof v);
@@ -1361,12 +1353,16 @@ struct lbm_mlp {
   long long woff[65], boff[65];  // offsets of W_l, b_l in the flat vector
   long long nparams;
   float *theta, *grad, *adam_m, *adam_v;
+  NetShape shape;
+  __nv_bfloat16 *fwd, *bwd;  // BF16 copies of the weights, behind theta (its allocation)
+  int net_rows;              // rows the training kernels of lbm_net.cuh take
   float* acts;         // activations: layer l input at acts + aoff[l]
   long long aoff[66];
-  float* dz[2];        // ping-pong backward buffers (max_batch x max width)
+  float* dz[2];        // ping-pong backward buffers (max_batch x max width); dz[0] also
+                       // holds dZ of every layer for net_rows rows
   float* dy;           // loss gradient (max_batch x n_out)
-  float* loss;         // device scalar
-  int* err;            // device error word of the GEMMs
+  float* loss;         // device scalar, then a partial sum per CTA of k_net_cluster
+  int* err;            // error word of the kernels (pinned host memory)
   long long step;
   cudaStream_t stream;
   char msg[512];
@@ -1400,7 +1396,7 @@ static void mlp_release(lbm_mlp* m) {
   lbm::dev_free(m->dz[1]);
   lbm::dev_free(m->dy);
   lbm::dev_free(m->loss);
-  lbm::dev_free(m->err);
+  lbm::host_free(m->err);
 }
 
 extern "C" lbm_status lbm_mlp_create(int n_in, int width, int depth, int n_out,
@@ -1439,29 +1435,39 @@ extern "C" lbm_status lbm_mlp_create(int n_in, int width, int depth, int n_out,
   }
   m->nparams = o;
   const size_t pb = sizeof(float) * (size_t)o;
+  m->shape = NetShape{n_in, width, depth, n_out};
+  m->net_rows = max_batch < kNetTrainRows ? max_batch : kNetTrainRows;
+  const size_t pack_at = (pb + 255) / 256 * 256;
+  const size_t pack_bytes = sizeof(__nv_bfloat16) * (size_t)m->shape.packed();
+  const size_t theta_bytes = pack_at + 2 * pack_bytes;
+  const size_t dz_all = (size_t)m->net_rows * ((size_t)depth * width + n_out);
   const size_t wmax = (size_t)max_batch * (size_t)(width > n_out ? (width > n_in ? width : n_in)
                                                                   : (n_out > n_in ? n_out : n_in));
   using lbm::dev_alloc;
-  bool okay = dev_alloc((void**)&m->theta, pb) == cudaSuccess &&
+  bool okay = dev_alloc((void**)&m->theta, theta_bytes) == cudaSuccess &&
               dev_alloc((void**)&m->grad, pb) == cudaSuccess &&
               dev_alloc((void**)&m->adam_m, pb) == cudaSuccess &&
               dev_alloc((void**)&m->adam_v, pb) == cudaSuccess &&
               dev_alloc((void**)&m->acts, sizeof(float) * (size_t)ao) == cudaSuccess &&
-              dev_alloc((void**)&m->dz[0], sizeof(float) * wmax) == cudaSuccess &&
+              dev_alloc((void**)&m->dz[0], sizeof(float) * (wmax > dz_all ? wmax : dz_all)) ==
+                  cudaSuccess &&
               dev_alloc((void**)&m->dz[1], sizeof(float) * wmax) == cudaSuccess &&
               dev_alloc((void**)&m->dy, sizeof(float) * (size_t)max_batch * n_out) == cudaSuccess &&
-              dev_alloc((void**)&m->loss, sizeof(float)) == cudaSuccess &&
-              dev_alloc((void**)&m->err, sizeof(int)) == cudaSuccess;
+              dev_alloc((void**)&m->loss, sizeof(float) * (1 + 8 * kNetTrainRows / kM)) ==
+                  cudaSuccess &&
+              lbm::host_alloc((void**)&m->err, sizeof(int)) == cudaSuccess;
   if (!okay) {
     cudaGetLastError();
     mlp_release(m);
     delete m;
     return mlp_fail(nullptr, LBM_ERR_OOM, "cudaMalloc failed");
   }
-  cudaMemsetAsync(m->theta, 0, pb, m->stream);
+  m->fwd = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(m->theta) + pack_at);
+  m->bwd = m->fwd + m->shape.packed();
+  cudaMemsetAsync(m->theta, 0, theta_bytes, m->stream);  // the copies' padding stays zero
   cudaMemsetAsync(m->adam_m, 0, pb, m->stream);
   cudaMemsetAsync(m->adam_v, 0, pb, m->stream);
-  cudaMemsetAsync(m->err, 0, sizeof(int), m->stream);
+  *m->err = 0;
   *out = m;
   return LBM_OK;
 }
@@ -1489,9 +1495,12 @@ extern "C" lbm_status lbm_mlp_set_params(lbm_mlp* m, const float* theta) {
            "cudaMemsetAsync");
   MLP_CUDA(m, cudaMemsetAsync(m->adam_v, 0, sizeof(float) * (size_t)m->nparams, m->stream),
            "cudaMemsetAsync");
-  // new parameters start a new history: a give-up reported before is cleared
-  MLP_CUDA(m, cudaMemsetAsync(m->err, 0, sizeof(int), m->stream), "cudaMemsetAsync");
+  k_net_pack<<<(unsigned)((m->nparams + 255) / 256), 256, 0, m->stream>>>(
+      m->shape, m->theta, m->nparams, m->fwd, m->bwd);
+  MLP_CUDA(m, cudaGetLastError(), "weight packing kernel");
   MLP_CUDA(m, cudaStreamSynchronize(m->stream), "stream sync");
+  // new parameters start a new history: a give-up reported before is cleared
+  *m->err = 0;
   m->step = 0;
   return LBM_OK;
 }
@@ -1547,13 +1556,50 @@ static lbm_status check_batch(lbm_mlp* m, int batch) {
   return LBM_OK;
 }
 
+// Waits for the stream; the error word lies in pinned host memory, which the
+// kernels write only when a wait gives up, so reading it needs no copy.
 static lbm_status check_err(lbm_mlp* m) {
-  int e = 0;
-  MLP_CUDA(m, cudaMemcpyAsync(&e, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream),
-           "cudaMemcpyAsync");
   MLP_CUDA(m, cudaStreamSynchronize(m->stream), "stream sync");
-  if (e) return mlp_fail(m, LBM_ERR_TIMEOUT, "a tensor-core GEMM wait gave up");
+  if (*(volatile int*)m->err)
+    return mlp_fail(m, LBM_ERR_TIMEOUT, "a tensor-core GEMM wait gave up");
   return LBM_OK;
+}
+
+// Whether the kernels may use the caller's array in place: device memory of
+// the current GPU, aligned to its floats.  Anything else goes through a copy.
+static bool in_place(const void* ptr) {
+  cudaPointerAttributes at;
+  int dev = -1;
+  if (((uintptr_t)ptr & 3u) != 0 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaPointerGetAttributes(&at, ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
+// The input rows where the kernels read them: x itself, or a copy in acts.
+static lbm_status net_input(lbm_mlp* m, const float* x, int batch, const float** out) {
+  *out = x;
+  if (in_place(x)) return LBM_OK;
+  MLP_CUDA(m, cudaMemcpyAsync(m->acts + m->aoff[0], x, sizeof(float) * (size_t)batch * m->n_in,
+                              cudaMemcpyDeviceToDevice, m->stream),
+           "cudaMemcpyAsync");
+  *out = m->acts + m->aoff[0];
+  return LBM_OK;
+}
+
+static NetArgs net_args(lbm_mlp* m, const float* x, int batch) {
+  NetArgs a;
+  memset(&a, 0, sizeof(a));
+  a.s = m->shape;
+  a.batch = batch;
+  a.x = x;
+  a.theta = m->theta;
+  a.fwd = m->fwd;
+  a.bwd = m->bwd;
+  a.err = m->err;
+  return a;
 }
 
 extern "C" lbm_status lbm_mlp_forward(lbm_mlp* m, const float* x, int batch, float* y) {
@@ -1561,16 +1607,60 @@ extern "C" lbm_status lbm_mlp_forward(lbm_mlp* m, const float* x, int batch, flo
   if (!m || !x || !y) return m ? mlp_fail(m, LBM_ERR_ARG, "NULL pointer") : LBM_ERR_ARG;
   lbm_status st = check_batch(m, batch);
   if (st != LBM_OK) return st;
-  float* yd = nullptr;
-  if ((st = mlp_forward_dev(m, x, batch, &yd)) != LBM_OK) return st;
-  MLP_CUDA(m, cudaMemcpyAsync(y, yd, sizeof(float) * (size_t)batch * m->n_out,
-                              cudaMemcpyDefault, m->stream),
-           "cudaMemcpyAsync");
-  return check_err(m);  // synchronises: a GEMM wait that gave up is reported
+  const float* xd = nullptr;
+  if ((st = net_input(m, x, batch, &xd)) != LBM_OK) return st;
+  const size_t xb = sizeof(float) * (size_t)batch * m->n_in;
+  const size_t yb = sizeof(float) * (size_t)batch * m->n_out;
+  // y may overlap x (its rows are then still inputs of other rows' CTAs)
+  const bool apart = (const char*)y + yb <= (const char*)xd || (const char*)xd + xb <= (const char*)y;
+  const bool direct = apart && in_place(y);
+  NetArgs a = net_args(m, xd, batch);
+  a.y = direct ? y : m->acts + m->aoff[m->nlayers];
+  MLP_CUDA(m, launch_net(a, m->stream), "network kernel launch");
+  if (!direct)
+    MLP_CUDA(m, cudaMemcpyAsync(y, a.y, yb, cudaMemcpyDefault, m->stream), "cudaMemcpyAsync");
+  return check_err(m);  // synchronises: a wait that gave up is reported
+}
+
+// Loss and gradient of up to net_rows rows: the forward pass, the loss and
+// the dZ chain of every 128 rows in one kernel, then every layer's weight and
+// bias gradient in another.
+static lbm_status net_backward(lbm_mlp* m, const float* x, const float* t, int batch) {
+  const float* xd = nullptr;
+  lbm_status st = net_input(m, x, batch, &xd);
+  if (st != LBM_OK) return st;
+  NetArgs a = net_args(m, xd, batch);
+  a.t = t;
+  a.scale = 1.f / (float)(batch * m->n_out);
+  a.h = m->acts + m->aoff[1];
+  a.h_stride = (long long)m->max_batch * m->width;
+  a.dz = m->dz[0];
+  a.dz_stride = (long long)m->net_rows * m->width;
+  a.loss_part = m->loss + 1;
+  MLP_CUDA(m, launch_net_cluster(a, m->stream), "network kernel launch");
+  DwArgs d;
+  memset(&d, 0, sizeof(d));
+  d.s = m->shape;
+  d.batch = batch;
+  d.x = xd;
+  d.h = a.h;
+  d.h_stride = a.h_stride;
+  d.dz = a.dz;
+  d.dz_stride = a.dz_stride;
+  d.grad = m->grad;
+  d.loss_part = a.loss_part;
+  const int c = net_cluster(m->shape), rows = net_rows_per_tile(batch, c);
+  d.loss_parts = (batch + rows - 1) / rows * c;
+  d.scale = a.scale;
+  d.loss = m->loss;
+  d.err = m->err;
+  MLP_CUDA(m, launch_net_dw(d, m->nparams, m->stream), "weight-gradient kernel launch");
+  return LBM_OK;
 }
 
 // Loss and gradient into m->grad (device).
 static lbm_status mlp_backward(lbm_mlp* m, const float* x, const float* t, int batch) {
+  if (batch <= m->net_rows) return net_backward(m, x, t, batch);
   float* y = nullptr;
   lbm_status st = mlp_forward_dev(m, x, batch, &y);
   if (st != LBM_OK) return st;
@@ -1655,9 +1745,10 @@ extern "C" lbm_status lbm_mlp_train_step(lbm_mlp* m, const float* x, const float
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = (float)(1.0 - pow(0.9, (double)m->step));
   const float c2 = (float)(1.0 - pow(0.999, (double)m->step));
-  k_adam<<<(unsigned)((m->nparams + 255) / 256), 256, 0, m->stream>>>(
-      m->theta, m->grad, m->adam_m, m->adam_v, m->nparams, lr, b1, b2, 1e-8f, c1, c2);
-  MLP_CUDA(m, cudaGetLastError(), "Adam kernel");
+  MLP_CUDA(m, launch_serial(k_net_adam, (unsigned)((m->nparams + 255) / 256), 1, 256, 0, 0,
+                            m->stream, m->shape, m->theta, m->grad, m->adam_m, m->adam_v,
+                            m->nparams, lr, b1, b2, 1e-8f, c1, c2, m->fwd, m->bwd),
+           "Adam kernel");
   if (loss) {
     MLP_CUDA(m, cudaMemcpyAsync(loss, m->loss, sizeof(float), cudaMemcpyDefault, m->stream),
              "cudaMemcpyAsync");

@@ -252,11 +252,12 @@ class Surrogate:
         """Normalised-space forward pass of device inputs, de-standardised."""
         n = Xd.shape[0]
         out = torch.empty((n, self.n_out), device=self.dev)
-        with torch.cuda.stream(self.stream):
-            for s in range(0, n, self.max_batch):
-                e = min(n, s + self.max_batch)
-                lbm.lbm_mlp_forward(self.m, Xd[s:e].contiguous(), e - s, out[s:e])
-        self.stream.synchronize()
+        if not Xd.is_contiguous():
+            with torch.cuda.stream(self.stream):
+                Xd = Xd.contiguous()
+        for s in range(0, n, self.max_batch):
+            e = min(n, s + self.max_batch)
+            lbm.lbm_mlp_forward(self.m, Xd[s:e], e - s, out[s:e])  # waits for its stream
         return out
 
     def predict(self, X: np.ndarray) -> np.ndarray:
