@@ -676,8 +676,7 @@ __device__ __forceinline__ bool tma_chunk(const T* __restrict__ src, T* __restri
   using Pair = typename Store<T>::Pair;
   unsigned char* stage0 = smem;
   float4(*win)[BY][TW] = reinterpret_cast<float4(*)[BY][TW]>(smem + NS * SB);
-  float(*hold)[BY - 2][TW - 2] =
-      reinterpret_cast<float(*)[BY - 2][TW - 2]>(smem + NS * SB + tma_win_bytes<TW, BY>());
+  unsigned char* hold = smem + NS * SB + tma_win_bytes<TW, BY>();
   unsigned long long* mbar = reinterpret_cast<unsigned long long*>(
       smem + NS * SB + tma_win_bytes<TW, BY>() + tma_hold_bytes<TW, BY>(HV));
 
@@ -687,6 +686,37 @@ __device__ __forceinline__ bool tma_chunk(const T* __restrict__ src, T* __restri
   const Geometry<WALLS, BY, TW> g(a, tx, ty, bx, by);
   const unsigned plane = (unsigned)a.plane;
   const Pair* srcp = reinterpret_cast<const Pair*>(src);
+  // the values an interior cell (thread tid < CELLS) holds from its pull to its
+  // collision, in the thread's own slots: [value / 4][cell] as float4, then the
+  // remaining ones as [value][cell]; 6 wide accesses each way instead of 24
+  constexpr int CELLS = (TW - 2) * (BY - 2), HQ = HV / 4;
+  float4* hold4 = reinterpret_cast<float4*>(hold);
+  float* hold1 = reinterpret_cast<float*>(hold + HQ * CELLS * 16);
+  auto put = [&](const float* f, const float* hu) {
+    auto val = [&](int i) { return i < 19 ? f[i] : hu[i - 19]; };
+#pragma unroll
+    for (int q = 0; q < HQ; ++q)
+      hold4[q * CELLS + tid] =
+          make_float4(val(4 * q), val(4 * q + 1), val(4 * q + 2), val(4 * q + 3));
+#pragma unroll
+    for (int i = 4 * HQ; i < HV; ++i) hold1[(i - 4 * HQ) * CELLS + tid] = val(i);
+  };
+  auto get = [&](float* f, float* hu) {
+    auto set = [&](int i, float v) {
+      if (i < 19) f[i] = v;
+      else hu[i - 19] = v;
+    };
+#pragma unroll
+    for (int q = 0; q < HQ; ++q) {
+      const float4 v = hold4[q * CELLS + tid];
+      set(4 * q, v.x);
+      set(4 * q + 1, v.y);
+      set(4 * q + 2, v.z);
+      set(4 * q + 3, v.w);
+    }
+#pragma unroll
+    for (int i = 4 * HQ; i < HV; ++i) set(i, hold1[(i - 4 * HQ) * CELLS + tid]);
+  };
   const int x0 = bx * (TW - 2), y0 = by * (BY - 2);
   // every source x - e_i, y - e_i of this column lies inside the lattice
   const bool col_fast = g.cx >= 1 && g.cx <= a.nx - 2 && g.cy >= 1 && g.cy <= a.ny - 2;
@@ -864,12 +894,7 @@ __device__ __forceinline__ bool tma_chunk(const T* __restrict__ src, T* __restri
     const bool got = tma_wait(mb(k), par(k), wait_ns);
     if (got) {
       fill(k, nf, nh);
-      if (g.interior) {  // private slot of this thread
-#pragma unroll
-        for (int i = 0; i < 19; ++i) hold[i][ty - 1][tx - 1] = nf[i];
-#pragma unroll
-        for (int i = 0; i < HV - 19; ++i) hold[19 + i][ty - 1][tx - 1] = nh[i];
-      }
+      if (g.interior) put(nf, nh);
     }
     if (!__syncthreads_and(got ? 1 : 0)) {
       drain(k);
@@ -891,10 +916,7 @@ __device__ __forceinline__ bool tma_chunk(const T* __restrict__ src, T* __restri
       const Recolour rc = collide_total<false>(a, cf, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
       store_recoloured<T>(dst, plane, a, (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1],
                           rc, cf);
-#pragma unroll
-      for (int i = 0; i < 19; ++i) cf[i] = hold[i][ty - 1][tx - 1];
-#pragma unroll
-      for (int i = 0; i < HV - 19; ++i) ch[i] = hold[19 + i][ty - 1][tx - 1];
+      get(cf, ch);
     }
     if constexpr (MON)
       if ((k - 2) % kMonFold == kMonFold - 1 || k == K - 1)
