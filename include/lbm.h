@@ -273,7 +273,8 @@ lbm_status lbm_set_planes(lbm_ctx *ctx, int z0, int n, const void *src);
    Batch contexts accept (tile_y, hold) = (8, 2), (8, 0), (16, 1) and, when
    every case has an x row of 16-byte multiple length, the TMA forms (8 or
    15, 7 or 8); their default is then (15, 32, 8) for FP32 and (15, 32, 7)
-   for 16-bit storage.
+   for 16-bit storage, or (12, 32, 7) or (8, 12, 2) where the boxes' tiles
+   make these cheaper.
    tile_y: CTA rows including the one-cell ring, 8 or 16 (the interior tile
    is 30 x (tile_y - 2) cells), or 15 (below).  zchunk: planes marched per CTA, 0 = the
    library's default for this lattice.  hold: where the populations of a

@@ -607,9 +607,8 @@ static lbm_status create_ctx(const lbm_params* ps, int ncases, void* cuda_stream
     delete[] hm;
     cudaGetLastError();
     // Batch default: the TMA form of the 34 x 15 tile, 32-plane chunks, one
-    // stage for FP32 and two for 16-bit storage (GB300, 512-case droplet
-    // sweep: 11.4 and 14.6 GLUPS against 10.0 and 12.5 for the 32 x 8
-    // shared-memory hold).
+    // stage for FP32 and two for 16-bit storage, unless another form is cheaper
+    // for the batch's boxes (batch_default_config)
     const int ns = c->storage == LBM_F32 ? 1 : 2;
     if (c->batch_tma_ok[2] && lbm::tma_config_fits(c->storage, 2, ns)) {
       c->fused.tile_y = 15;
@@ -636,12 +635,13 @@ static lbm_status create_ctx(const lbm_params* ps, int ncases, void* cuda_stream
     }
     delete[] hs;
     cudaGetLastError();
-    // an option for the autotuner, not the default: on the 512-case droplet
-    // sweep (GB300) the 34 x 15 one-stage form above runs 11.5 ms per step
-    // against 13.5 ms for this one at its best chunk (48 planes): most of
-    // the sweep's cells are in 96^3 cases, whose 34 x 12 tiles are ragged
-    // in y and carry more ring per cell
     c->batch_seam_ok = seam;
+    const StepArgs** args = new (std::nothrow) const StepArgs*[(size_t)ncases];
+    if (args && c->fused.tile_y == 15 && !c->cases[0].args.bgk) {
+      for (int k = 0; k < ncases; ++k) args[k] = &c->cases[k].args;
+      lbm::batch_default_config(args, ncases, c->storage, c->sms, seam, &c->fused);
+    }
+    delete[] args;
   }
   if (st == LBM_OK && ncases > 1 &&
       lbm::dev_alloc((void**)&c->d_cases, sizeof(lbm::BatchCase) * ncases) != cudaSuccess)

@@ -314,6 +314,78 @@ bool valid_batch_config(const FusedConfig& c) {
   return shape && c.zchunk > 0;
 }
 
+// A batch's CTAs in one form of the step: places (SMs x CTAs per SM), and when
+// the last CTA ends, in plane-times.  The CTAs are handed out in launch order
+// to the place that falls free first; past 8192 of them the schedule is taken
+// as their work over the places and half a CTA's for the ragged end.
+namespace {
+class BatchSpan {
+ public:
+  explicit BatchSpan(int places) : free_((size_t)places, 0.0) {}
+  void add(const StepArgs& a, int iw, int ih, int zc, double overhead) {
+    const long long tiles = (long long)((a.nx + iw - 1) / iw) * ((a.ny + ih - 1) / ih);
+    for (int z = 0; z < a.nz; z += zc) {
+      const double d = std::min(zc, a.nz - z) + overhead;
+      longest_ = std::max(longest_, d);
+      work_ += (double)tiles * d;
+      if ((items_ += tiles) > 8192) continue;
+      auto later = std::greater<double>();
+      for (long long t = 0; t < tiles; ++t) {
+        std::pop_heap(free_.begin(), free_.end(), later);
+        free_.back() += d;
+        end_ = std::max(end_, free_.back());
+        std::push_heap(free_.begin(), free_.end(), later);
+      }
+    }
+  }
+  long long items() const { return items_; }
+  double end() const {
+    return items_ > 8192 ? work_ / (double)free_.size() + 0.5 * longest_ : end_;
+  }
+
+ private:
+  std::vector<double> free_;
+  long long items_ = 0;
+  double work_ = 0.0, longest_ = 0.0, end_ = 0.0;
+};
+}  // namespace
+
+// Which form a batch runs: the one whose schedule ends first, a plane-time
+// taking 3.75 us on the 34 x 15 tile (its seam lanes pull from global memory),
+// 2.75 us on the 34 x 12 seam form and 2.85 us on the 32 x 8 tile with two CTAs
+// per SM.  GB300, us per step in these three, FP32: 128 boxes of 64 x 64 x 32
+// with a floor 1226 / 1140 / 1657; 60 of 64 x 64 x 24 426 / 456 / 557; 60 of 40 x
+// 40 x 24 367 / 304 / 242; 60 of 48 x 51 x 37 562 / 647 / 493; 60 of 96 x 40 x 32
+// 624 / 502 / 649; 60 of 96 x 64 x 24 602 / 657 / 752; 48 droplet boxes of 32 to
+// 96 cells 1268 / 1535 / 1481; 16 bits, 34 x 15 / 32 x 8: 60 of 40 x 40 x 24 326 /
+// 241, 60 of 64 x 72 x 32 670 / 812.  The seam form only where no box is narrower
+// than its tile (the droplet boxes' 32-cell ones are what slows it there).  A
+// batch of fewer than 32 CTAs keeps the tensor-copy form, whose bounded waits
+// the fault tests step.
+void batch_default_config(const StepArgs* const* args, int ncases, int storage, int sms,
+                          bool seam_ok, FusedConfig* c) {
+  BatchSpan t15(sms), t12(sms), t8(2 * sms);
+  bool seam = storage == 0 && seam_ok;
+  for (int k = 0; k < ncases; ++k) {
+    const StepArgs& a = *args[k];
+    t15.add(a, 32, 13, 32, 3.0);
+    t12.add(a, 32, 10, 32, 3.0);
+    t8.add(a, 30, 6, 12, 2.5);
+    seam = seam && a.nx >= kTmaTW[2] && a.ny >= kTmaBY[2];
+  }
+  if (t15.items() < 32) return;
+  const double c15 = 3.75 * t15.end(), c12 = 2.75 * t12.end(), c8 = 2.85 * t8.end();
+  if (seam && c12 < c15 && c12 <= c8) {
+    c->tile_y = 12;
+    c->zchunk = 32;
+    c->hold = 7;
+  } else if (c8 < c15) {
+    c->tile_y = 8;
+    c->zchunk = 12;
+    c->hold = 2;
+  }
+}
+
 bool batch_seam_eligible(const StepArgs& a, int storage) {
   return storage == 0 && tma_eligible(a, storage) && !a.wx && !a.wy && !a.bgk;
 }

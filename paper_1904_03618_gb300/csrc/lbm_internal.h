@@ -239,6 +239,10 @@ cudaError_t launch_fused_tma_batch(int storage, const void* src, void* dst,
                                    bool walls, const CUtensorMap* maps, int kind, int ns, int zc,
                                    int* err, int sms, cudaStream_t s);
 bool valid_batch_config(const FusedConfig& c);
+// Replaces the 34 x 15 tensor-copy default *c of a batch where another form is
+// cheaper (seam_ok: the batched SEAM form's maps were built).
+void batch_default_config(const StepArgs* const* args, int ncases, int storage, int sms,
+                          bool seam_ok, FusedConfig* c);
 // Batched SEAM step: maps6 = the device table of the source buffer's six
 // seam maps (tile_y 12) per case.
 cudaError_t launch_fused_tma_seam_batch(const void* src, void* dst, const BatchCase* cases,
