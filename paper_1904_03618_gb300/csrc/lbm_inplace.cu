@@ -41,7 +41,15 @@
 namespace lbm {
 namespace {
 
-constexpr int kInplaceBlock = 128;
+constexpr int kInplaceBlock = 128;  // threads per block at most
+// Threads per block: the rows' cells in as few warps as 128, 96 or 64 threads
+// allow.
+int block_threads(int nx) {
+  int best = kInplaceBlock;
+  for (int t : {96, 64})
+    if ((nx + t - 1) / t * t < (nx + best - 1) / best * best) best = t;
+  return best;
+}
 
 struct Site {
   int x, y, z;
@@ -173,42 +181,123 @@ __global__ void __launch_bounds__(kInplaceBlock)
   }
 }
 
+// The step's own addressing.  A block is a piece of one row, so the row and
+// plane parts of every neighbour's index, and the walls beyond them, are the
+// same for all its threads: an access costs one add (the thread's x part onto a
+// block-uniform base) and the address.  Idx: 32 bits while 38 N fits them (up
+// to 113 million cells), else 64.  WALLS = false: periodic lattices.
+template <typename Idx, bool WALLS>
+struct Rows {
+  Idx x[3], row[3][3], N;       // x + d; the row of (y + dy, z + dz), [dy + 1][dz + 1]
+  bool xb[3], yb[3], zb[3];     // beyond a wall
+  __device__ __forceinline__ Rows(const StepArgs& a, const Site& s, long long n) : N((Idx)n) {
+    Idx yo[3], zo[3];
+    const Idx plane = (Idx)a.nx * (Idx)a.ny;
+#pragma unroll
+    for (int d = -1; d <= 1; ++d) {
+      const int xn = s.x + d, yn = s.y + d, zn = s.z + d;
+      xb[d + 1] = WALLS && a.wx && (xn < 0 || xn >= a.nx);
+      yb[d + 1] = WALLS && a.wy && (yn < 0 || yn >= a.ny);
+      zb[d + 1] = WALLS && a.wz && (zn < 0 || zn >= a.nz);
+      x[d + 1] = (Idx)wrap1(xn, a.nx);
+      yo[d + 1] = (Idx)wrap1(yn, a.ny) * (Idx)a.nx;
+      zo[d + 1] = (Idx)wrap1(zn, a.nz) * plane;
+    }
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+      for (int dz = 0; dz < 3; ++dz) row[dy][dz] = yo[dy] + zo[dz];
+  }
+  __device__ __forceinline__ Idx cell(int dx, int dy, int dz) const {
+    return row[dy + 1][dz + 1] + x[dx + 1];
+  }
+  __device__ __forceinline__ bool beyond(int dx, int dy, int dz) const {
+    return WALLS && (xb[dx + 1] || yb[dy + 1] || zb[dz + 1]);
+  }
+  // Forgets where the indices came from, so that the store addresses are formed
+  // anew instead of the loads' 38 being kept in registers over the collision
+  // (144 bytes of spills in the odd form).
+  __device__ __forceinline__ void refresh() {
+    auto opaque = [](Idx& v) {
+      if constexpr (sizeof(Idx) == 4) asm volatile("" : "+r"(v));
+      else asm volatile("" : "+l"(v));
+    };
+#pragma unroll
+    for (int d = 0; d < 3; ++d) opaque(x[d]);
+    if (!WALLS || sizeof(Idx) == 8) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) opaque(row[k / 3][k % 3]);
+    }
+  }
+  // Offset, within one colour, of the slot that holds f_i(x, t).
+  template <int ODD>
+  __device__ __forceinline__ Idx slot(int i) const {
+    if (!ODD) return (Idx)i * N + cell(0, 0, 0);
+    const int dx = -ex(i), dy = -ey(i), dz = -ez(i);
+    const Idx in = ((Idx)opp(i) * N + row[dy + 1][dz + 1]) + x[dx + 1];
+    if (!WALLS) return in;
+    return beyond(dx, dy, dz) ? ((Idx)i * N + row[1][1]) + x[1] : in;
+  }
+};
+
+// The populations of the cell, reduced to (f_i = fR_i + fB_i, rho_R, rho_B).
+template <int ODD, typename T, typename R>
+__device__ __forceinline__ void load_total(const T* fr, const T* fb, const StepArgs& a, const R& n,
+                                           float* f, float& rR, float& rB) {
+  rR = 0.f;
+  rB = 0.f;
+#pragma unroll
+  for (int i = 0; i < 19; ++i) {
+    const auto o = n.template slot<ODD>(i);
+    const float r = ip_load(fr + o, a, 0, i), b = ip_load(fb + o, a, 1, i);
+    rR += r;
+    rB += b;
+    f[i] = r + b;
+  }
+}
+
 // Pass 1: (rho^N, Qbar) of every cell at time t.
-template <int ODD, typename T>
+template <int ODD, typename Idx, bool WALLS, typename T>
 __global__ void __launch_bounds__(kInplaceBlock)
     k_inplace_phase(const T* __restrict__ f, StepArgs a, long long N,
                     float4* __restrict__ phase) {
   Site s;
   if (!site_of(a, s)) return;
-  const Nbr nb = neighbourhood(a, s);
-  float fR[19], fB[19];
-  load_site<ODD>(f, a, nb, s, N, fR, fB);
-  phase[s.c] = stencil_entry(a, macro_of(a, fR, fB));
+  const Rows<Idx, WALLS> n(a, s, N);
+  float ft[19], rR, rB;
+  load_total<ODD>(f, f + 19 * N, a, n, ft, rR, rB);
+  phase[n.cell(0, 0, 0)] = stencil_entry(a, macro_total(a, ft, rR, rB));
 }
 
 // Pass 2: Eq. 49 gradients from the phase field (a neighbour beyond a wall
 // takes the cell's own entry), collision, perturbation and recolouring, and
 // the in-place write.  f is read and written by this kernel: plain loads.
-// Four blocks per SM (at most 128 registers, 16 warps; the odd form spills
-// 16 bytes): 7 % faster than the 139-144 registers and 12 warps the
-// compiler picks unbounded.
-template <int ODD, bool BGK, typename T>
+// Four 128-thread blocks' registers per SM (128 a thread, 16 warps): three
+// blocks 192 us a step at 128^3, four 187, five 231 (spills).  What bounds it:
+// the loads' latency at 16 warps, about 5 TB/s of its 320 B per cell; the
+// instructions were the rest -- with 64-bit indices formed per thread, walls
+// tested per access and the loads' addresses kept for the stores, 128^3 took 217
+// us, 192 x 192 x 768 3020 (now 2576, of which the 64-thread blocks of its
+// 192-cell rows 8 %), 131^3 292 (232).  Tried on top and dropped: the phase
+// field of the next slab of planes in the launch of this slab's collision, to
+// find its populations in L2 (192 x 192 x 768 2890 at the best slab, 128^3 185).
+template <int ODD, bool BGK, typename Idx, bool WALLS, typename T>
 __global__ void __launch_bounds__(kInplaceBlock, 4)
     k_inplace_collide(T* f, StepArgs a, long long N, const float4* __restrict__ phase) {
   Site s;
   if (!site_of(a, s)) return;
-  const Nbr nb = neighbourhood(a, s);
-  float fR[19], fB[19];
-  load_site<ODD>(f, a, nb, s, N, fR, fB);
-  const Macro m = macro_of(a, fR, fB);
-  const float4 ctr = phase[s.c];
+  Rows<Idx, WALLS> n(a, s, N);
+  T* const fb = f + 19 * N;
+  float ft[19], rR, rB;
+  load_total<ODD>(f, fb, a, n, ft, rR, rB);
+  const Macro m = macro_total(a, ft, rR, rB);
+  const float4 ctr = phase[n.cell(0, 0, 0)];
   float Gx = 0.f, Gy = 0.f, Gz = 0.f, Qx = 0.f, Qy = 0.f, Qz = 0.f;
 #pragma unroll
   for (int i = 1; i < 19; i += 2) {
-    const long long np = site_shift(nb, ex(i), ey(i), ez(i));
-    const long long nm = site_shift(nb, -ex(i), -ey(i), -ez(i));
-    const float4 vp = np < 0 ? ctr : phase[np];
-    const float4 vm = nm < 0 ? ctr : phase[nm];
+    float4 vp = ctr, vm = ctr;
+    if (!n.beyond(ex(i), ey(i), ez(i))) vp = phase[n.cell(ex(i), ey(i), ez(i))];
+    if (!n.beyond(-ex(i), -ey(i), -ez(i))) vm = phase[n.cell(-ex(i), -ey(i), -ez(i))];
     const float w = (i <= 6) ? (1.0f / 6.0f) : (1.0f / 12.0f);
     if (ex(i)) {
       Gx += (ex(i) * w) * (vp.x - vm.x);
@@ -223,16 +312,19 @@ __global__ void __launch_bounds__(kInplaceBlock, 4)
       Qz += (ez(i) * w) * (vp.w - vm.w);
     }
   }
-  if (a.wetting)
+  if (WALLS && a.wetting)
     wetting_rule(a, a.wx && s.x == 0, a.wx && s.x == a.nx - 1, a.wy && s.y == 0,
                  a.wy && s.y == a.ny - 1, a.wz && s.z == 0, a.wz && s.z == a.nz - 1, Gx, Gy,
                  Gz);
-  collide_cell<BGK>(a, fR, fB, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+  const Recolour rc = collide_total<BGK>(a, ft, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+  float fR[19], fB[19];
+  RecolourAll<0>::run(rc, ft, fR, fB);
+  n.refresh();
 #pragma unroll
   for (int i = 0; i < 19; ++i) {
-    const long long o = slot_of<ODD>(nb, s, opp(i), N);
+    const auto o = n.template slot<ODD>(opp(i));
     ip_store(f + o, fR[i], a, 0, i);
-    ip_store(f + 19 * N + o, fB[i], a, 1, i);
+    ip_store(fb + o, fB[i], a, 1, i);
   }
 }
 
@@ -302,24 +394,31 @@ cudaError_t ip_set(const lbm_params* p, const StepArgs& a, long long N, void* f,
   k_inplace_set<T><<<site_grid(p), kInplaceBlock, 0, s>>>((T*)f, a, N, f_in);
   return cudaGetLastError();
 }
+template <int ODD, bool BGK, typename Idx, bool WALLS, typename T>
+void ip_passes(const StepArgs& a, long long N, T* f, float4* phase, cudaStream_t s) {
+  const int t = block_threads(a.nx);
+  const dim3 g((unsigned)((a.nx + t - 1) / t), (unsigned)a.ny, (unsigned)a.nz);
+  k_inplace_phase<ODD, Idx, WALLS, T><<<g, t, 0, s>>>(f, a, N, phase);
+  k_inplace_collide<ODD, BGK, Idx, WALLS, T><<<g, t, 0, s>>>(f, a, N, phase);
+}
+
+template <int ODD, typename T>
+void ip_parity(const StepArgs& a, long long N, T* f, float4* phase, cudaStream_t s) {
+  using U64 = unsigned long long;
+  if (38 * N >= (1LL << 32))
+    a.bgk ? ip_passes<ODD, true, U64, true, T>(a, N, f, phase, s)
+          : ip_passes<ODD, false, U64, true, T>(a, N, f, phase, s);
+  else if (a.bgk) ip_passes<ODD, true, unsigned, true, T>(a, N, f, phase, s);
+  else if (a.wx || a.wy || a.wz) ip_passes<ODD, false, unsigned, true, T>(a, N, f, phase, s);
+  else ip_passes<ODD, false, unsigned, false, T>(a, N, f, phase, s);
+}
+
 template <typename T>
 cudaError_t ip_step(const lbm_params* p, const StepArgs& a, long long N, void* fv, int parity,
                     float4* phase, cudaStream_t s) {
-  T* f = (T*)fv;
-  const dim3 g = site_grid(p);
-  if (parity) {
-    k_inplace_phase<1, T><<<g, kInplaceBlock, 0, s>>>(f, a, N, phase);
-    if (a.bgk)
-      k_inplace_collide<1, true, T><<<g, kInplaceBlock, 0, s>>>(f, a, N, phase);
-    else
-      k_inplace_collide<1, false, T><<<g, kInplaceBlock, 0, s>>>(f, a, N, phase);
-  } else {
-    k_inplace_phase<0, T><<<g, kInplaceBlock, 0, s>>>(f, a, N, phase);
-    if (a.bgk)
-      k_inplace_collide<0, true, T><<<g, kInplaceBlock, 0, s>>>(f, a, N, phase);
-    else
-      k_inplace_collide<0, false, T><<<g, kInplaceBlock, 0, s>>>(f, a, N, phase);
-  }
+  (void)p;
+  if (parity) ip_parity<1, T>(a, N, (T*)fv, phase, s);
+  else ip_parity<0, T>(a, N, (T*)fv, phase, s);
   return cudaGetLastError();
 }
 template <typename T>
