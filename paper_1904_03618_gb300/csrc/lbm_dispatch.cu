@@ -419,17 +419,18 @@ FusedConfig default_fused_config(const StepArgs& a, int storage) {
   return c;
 }
 
-// The box form's range, GB300, us per step (box / marching kernel): it wins
-// up to about 260,000 cells (FP32 56^3 16.3 / 25.0, 64^3 24.2 / 27.6, 80^3
-// 48 / 43; FP16 64^3 21.5 / 28.7; 65 x 64 x 64 with walls 35 / 36).  On the
-// lattices of the seam forms, the line lies lower than that, at 81,920
+// The box form's range, GB300, us per step (box / the fastest marching chunk):
+// with walls 45^3 11.3 / 16.5, 59^3 21.3 / 20.6, 60^3 20.7 / 18.5; FP16 45^3 9.6 /
+// 13.3, 59^3 18.7 / 17.4; BGK 45^3 10.3 / 14.3, 59^3 20.0 / 17.4, 120 x 70 x 29
+// FP16 21.3 / 18.9; 101 x 50 x 50 25.3 / 20.5: it wins up to about 180,000 cells.
+// On the lattices of the seam forms, the line lies lower than that, at 81,920
 // cells: from there on the tensor-copy kernel with its bounded waits, which
 // reports them in the error word, is the documented default (the fault tests
 // step a 64 x 40 x 36 lattice through it).
 int default_box(const StepArgs& a, int storage) {
   const long long N = (long long)a.nx * a.ny * a.nz;
   const bool seam = seam_eligible(a, storage) || seam16_eligible(a, storage);
-  if (N > (seam ? 81920 : 262144)) return 0;
+  if (N > (seam ? 81920 : 180000)) return 0;
   return N <= 16384 ? 1 : 2;
 }
 
