@@ -38,10 +38,8 @@ constexpr int kTileW = 32;  // threads along x per CTA (one warp)
 
 template <typename T, int I>
 __device__ __forceinline__ void add_offsets(const StepArgs& a, float2& v) {
-  if (Store<T>::kDeviation) {
-    v.x += dev_offset<I>(a, 0);
-    v.y += dev_offset<I>(a, 1);
-  }
+  if (Store<T>::kDeviation)
+    v = __fadd2_rn(v, make_float2(dev_offset<I>(a, 0), dev_offset<I>(a, 1)));
 }
 
 // Pull of the 19 pairs of one column / plane, reduced on the fly to
@@ -123,9 +121,10 @@ struct PullAsync<T, WALLS, 19> {
 // opposite directions at a time (their recolouring terms differ in sign).
 template <typename T, int I>
 struct StoreRecoloured {
+  template <typename Rc>
   __device__ __forceinline__ static void run(T* dst, unsigned plane,
                                              const StepArgs& a, unsigned c,
-                                             const Recolour& rc,
+                                             const Rc& rc,
                                              const float* fs) {
     const float sg = recolour_seg<I>(rc);
     float r1 = rc.wr * fs[I] + sg, b1 = rc.wb * fs[I] - sg;
@@ -143,14 +142,15 @@ struct StoreRecoloured {
 };
 template <typename T>
 struct StoreRecoloured<T, 19> {
+  template <typename Rc>
   __device__ __forceinline__ static void run(T*, unsigned, const StepArgs&,
-                                             unsigned, const Recolour&,
+                                             unsigned, const Rc&,
                                              const float*) {}
 };
-template <typename T>
+template <typename T, typename Rc>
 __device__ __forceinline__ void store_recoloured(T* dst, unsigned plane,
                                                  const StepArgs& a, unsigned c,
-                                                 const Recolour& rc,
+                                                 const Rc& rc,
                                                  const float* fs) {
   if (!index_ok(a, c, plane)) return;
   float r0 = rc.wr * fs[0], b0 = rc.wb * fs[0];
@@ -362,7 +362,7 @@ __device__ __forceinline__ void fused_work(const T* __restrict__ src,
       } else {
         m = macro_held(a, ch[0], ch[1], ch[2], ch[3], ch[4]);
       }
-      const Recolour rc = collide_total<BGK>(a, cf, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+      const auto rc = collide_stored<T, BGK>(a, cf, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
       store_recoloured<T>(dst, plane, a,
                           (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1], rc, cf);
     }
@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(kTileW * 8, 2)
     const Macro m = macro_held(a, h[19][row - 1][tx - 1], h[20][row - 1][tx - 1],
                                h[21][row - 1][tx - 1], h[22][row - 1][tx - 1],
                                h[23][row - 1][tx - 1]);
-    const Recolour rc = collide_total<false>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+    const auto rc = collide_stored<T>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
     store_recoloured<T>(dst, plane, a, (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1],
                         rc, f);
   };
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kTileW* kAsyncBY, 2)
       for (int i = 0; i < 19; ++i) f[i] = h[i * hs];
       const Macro m = macro_held(a, h[19 * hs], h[20 * hs], h[21 * hs], h[22 * hs],
                                  h[23 * hs]);
-      const Recolour rc = collide_total<false>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+      const auto rc = collide_stored<T>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
       store_recoloured<T>(dst, plane, a,
                           (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1], rc, f);
     }
