@@ -626,15 +626,13 @@ __device__ __forceinline__ Recolour collide_total(const StepArgs& a, float* f,
 // The same collision with fewer operations (about a tenth of the step's): the
 // residuals m^eq - m from shared products (rho u_a u_b, A = rho |u|^2), sources
 // only where there are any, recolouring terms formed once per axis.  Its
-// results differ from collide_total's in the last bits (errors against a 64-bit
-// run are the same), so it runs where nothing is held to those bits: in 16-bit
-// storage, whose stores round 10^4 times more coarsely, in the in-place step,
-// and in single FP32 lattices without walls in x or y.  (Others keep
-// collide_total's bits: drops at relaxation times near 1/2 multiply a changed
-// last bit a thousandfold within 24 steps.)  GB300, us per step: 192 x 192 x 768
-// BF16 1553 -> 1500, FP16 droplet sweep 1189 -> 1150, 128^3 FP16 121.1 -> 120.0, in
-// place 192 x 192 x 768 FP32 2675 -> 2641; FP32 256 x 256 x 1024 3642 -> 3559,
-// 128^3 131.3 -> 129.8.
+// results differ from collide_total's in the last bits, so it runs where nothing
+// is held to those bits: in 16-bit storage, whose stores round 10^4 times more
+// coarsely, and in the in-place step.  (FP32 steps keep collide_total's bits:
+// drops at relaxation times near 1/2 multiply a changed last bit a thousandfold
+// within 24 steps.)  GB300, us per step: 192 x 192 x 768 BF16 1553 -> 1500, FP16
+// droplet sweep 1189 -> 1150, 128^3 FP16 121.1 -> 120.0, in place 192 x 192 x 768
+// FP32 2675 -> 2641.
 // ---------------------------------------------------------------------------
 struct RecolourLean {
   float wr, wb;
@@ -832,12 +830,12 @@ __device__ __forceinline__ RecolourLean collide_lean(const StepArgs& a, float* f
   return collide_post<BGK>(a, f, R, mc, rhoN, Gx, Gy, Gz, Qx, Qy, Qz);
 }
 
-// The one a kernel runs.
-template <bool LEAN, bool BGK = false>
-__device__ __forceinline__ auto collide_as(const StepArgs& a, float* f, const Macro& mc,
-                                           float rhoN, float Gx, float Gy, float Gz, float Qx,
-                                           float Qy, float Qz) {
-  if constexpr (LEAN)
+// The collision a kernel of storage type T runs.
+template <typename T, bool BGK = false>
+__device__ __forceinline__ auto collide_stored(const StepArgs& a, float* f, const Macro& mc,
+                                               float rhoN, float Gx, float Gy, float Gz, float Qx,
+                                               float Qy, float Qz) {
+  if constexpr (Store<T>::kDeviation)
     return collide_lean<BGK>(a, f, mc, rhoN, Gx, Gy, Gz, Qx, Qy, Qz);
   else
     return collide_total<BGK>(a, f, mc, rhoN, Gx, Gy, Gz, Qx, Qy, Qz);

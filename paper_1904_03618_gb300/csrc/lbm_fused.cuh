@@ -36,16 +36,6 @@ namespace lbm {
 
 constexpr int kTileW = 32;  // threads along x per CTA (one warp)
 
-// Whether a single lattice's default forms run the lean collision: always in
-// 16-bit storage, in FP32 unless there are walls in x or y (closed boxes of
-// drops at relaxation times near 1/2 keep collide_total's bits, as do FP32
-// batches of them).  All forms of one lattice decide alike, so that a slab of it
-// steps as the whole does, whichever form each runs.
-template <typename T>
-inline bool lean_collision(const StepArgs& a) {
-  return Store<T>::kDeviation || (!a.wx && !a.wy);
-}
-
 template <typename T, int I>
 __device__ __forceinline__ void add_offsets(const StepArgs& a, float2& v) {
   if (Store<T>::kDeviation)
@@ -313,8 +303,7 @@ __device__ __forceinline__ void hold_get(const Slot& slot, float* f, float* hu) 
 
 // MINB: CTAs per SM the register allocation must allow (launch bounds).
 // One work item of the fused step: tile (bx, by), planes [zb, ze).
-template <typename T, int BY, bool WALLS, int HOLD, bool BGK = false,
-          bool LEAN = Store<T>::kDeviation>
+template <typename T, int BY, bool WALLS, int HOLD, bool BGK = false>
 __device__ __forceinline__ void fused_work(const T* __restrict__ src,
                                            T* __restrict__ dst,
                                            const StepArgs& a, int bx, int by,
@@ -373,7 +362,7 @@ __device__ __forceinline__ void fused_work(const T* __restrict__ src,
       } else {
         m = macro_held(a, ch[0], ch[1], ch[2], ch[3], ch[4]);
       }
-      const auto rc = collide_as<LEAN, BGK>(a, cf, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+      const auto rc = collide_stored<T, BGK>(a, cf, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
       store_recoloured<T>(dst, plane, a,
                           (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1], rc, cf);
     }
@@ -389,8 +378,7 @@ __device__ __forceinline__ void fused_work(const T* __restrict__ src,
   }
 }
 
-template <typename T, int BY, bool WALLS, int HOLD, int MINB, bool BGK = false,
-          bool LEAN = Store<T>::kDeviation>
+template <typename T, int BY, bool WALLS, int HOLD, int MINB, bool BGK = false>
 __global__ void __launch_bounds__(kTileW* BY, MINB)
     k_fused(const T* __restrict__ src, T* __restrict__ dst,
             const __grid_constant__ StepArgs a, int zchunk) {
@@ -398,7 +386,7 @@ __global__ void __launch_bounds__(kTileW* BY, MINB)
   const int zb = blockIdx.z * zchunk;
   const int ze = min(zb + zchunk, a.nz);
   if (zb >= ze) return;
-  fused_work<T, BY, WALLS, HOLD, BGK, LEAN>(src, dst, a, blockIdx.x, blockIdx.y, zb, ze, sm);
+  fused_work<T, BY, WALLS, HOLD, BGK>(src, dst, a, blockIdx.x, blockIdx.y, zb, ze, sm);
 }
 
 // Batched step: many independent lattices ("cases") in one launch.  The
@@ -506,7 +494,7 @@ __global__ void __launch_bounds__(kTileW * 8, 2)
     const Macro m = macro_held(a, h[19][row - 1][tx - 1], h[20][row - 1][tx - 1],
                                h[21][row - 1][tx - 1], h[22][row - 1][tx - 1],
                                h[23][row - 1][tx - 1]);
-    const auto rc = collide_as<Store<T>::kDeviation>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+    const auto rc = collide_stored<T>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
     store_recoloured<T>(dst, plane, a, (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1],
                         rc, f);
   };
@@ -620,7 +608,7 @@ __global__ void __launch_bounds__(kTileW* kAsyncBY, 2)
       for (int i = 0; i < 19; ++i) f[i] = h[i * hs];
       const Macro m = macro_held(a, h[19 * hs], h[20 * hs], h[21 * hs], h[22 * hs],
                                  h[23 * hs]);
-      const auto rc = collide_as<Store<T>::kDeviation>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+      const auto rc = collide_stored<T>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
       store_recoloured<T>(dst, plane, a,
                           (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1], rc, f);
     }
@@ -630,14 +618,13 @@ __global__ void __launch_bounds__(kTileW* kAsyncBY, 2)
 }
 
 template <typename T, int BY, bool WALLS, int HOLD,
-          int MINB = (BY == 8 && HOLD != 1) ? 2 : 1, bool BGK = false,
-          bool LEAN = Store<T>::kDeviation>
+          int MINB = (BY == 8 && HOLD != 1) ? 2 : 1, bool BGK = false>
 static cudaError_t launch_fused_v(const void* src, void* dst,
                                   const StepArgs& a, int zc, cudaStream_t s) {
   dim3 blk(kTileW, BY);
   dim3 grd((a.nx + kTileW - 3) / (kTileW - 2), (a.ny + BY - 3) / (BY - 2),
            (a.nz + zc - 1) / zc);
-  k_fused<T, BY, WALLS, HOLD, MINB, BGK, LEAN><<<grd, blk, 0, s>>>((const T*)src, (T*)dst, a, zc);
+  k_fused<T, BY, WALLS, HOLD, MINB, BGK><<<grd, blk, 0, s>>>((const T*)src, (T*)dst, a, zc);
   return cudaGetLastError();
 }
 
@@ -680,16 +667,6 @@ static cudaError_t launch_fused2(const void* src, void* dst, const StepArgs& a,
   return cudaGetLastError();
 }
 
-// The default form: the collision the lattice's other default forms run.
-template <typename T, bool WALLS, bool BGK>
-static cudaError_t launch_fused_hold2(const void* src, void* dst, const StepArgs& a, int zc,
-                                      cudaStream_t s) {
-  if constexpr (WALLS && !Store<T>::kDeviation)
-    if (!lean_collision<T>(a))
-      return launch_fused_v<T, 8, WALLS, 2, 2, BGK, false>(src, dst, a, zc, s);
-  return launch_fused_v<T, 8, WALLS, 2, 2, BGK, true>(src, dst, a, zc, s);
-}
-
 template <typename T, int BY, bool WALLS>
 static cudaError_t launch_fused_h(const void* src, void* dst,
                                   const StepArgs& a, const FusedConfig& cfg,
@@ -699,7 +676,7 @@ static cudaError_t launch_fused_h(const void* src, void* dst,
     case 1: return launch_fused_v<T, BY, WALLS, 1>(src, dst, a, zc, s);
     case 2:
       // the shared-memory hold fits the 48 KB static limit only for BY = 8
-      if constexpr (BY == 8) return launch_fused_hold2<T, WALLS, false>(src, dst, a, zc, s);
+      if constexpr (BY == 8) return launch_fused_v<T, BY, WALLS, 2>(src, dst, a, zc, s);
       break;
     case 3:
       if constexpr (BY == 8) return launch_fused_async<T, WALLS>(src, dst, a, zc, s);
@@ -772,8 +749,8 @@ cudaError_t launch_fused_storage(const void* src, void* dst,
   const bool walls = a.wx || a.wy || a.wz;
   if (a.bgk) {  // the BGK operator runs the shared-memory-hold form only
     if (cfg.tile_y != 8 || cfg.hold != 2) return cudaErrorInvalidValue;
-    return walls ? launch_fused_hold2<T, true, true>(src, dst, a, zc, s)
-                 : launch_fused_hold2<T, false, true>(src, dst, a, zc, s);
+    return walls ? launch_fused_v<T, 8, true, 2, 2, true>(src, dst, a, zc, s)
+                 : launch_fused_v<T, 8, false, 2, 2, true>(src, dst, a, zc, s);
   }
   if (cfg.tile_y == 8)
     return walls ? launch_fused_h<T, 8, true>(src, dst, a, cfg, zc, s)

@@ -66,7 +66,7 @@ struct BoxShape {
   }
 };
 
-template <typename T, int BX, int BY, int BZ, bool WALLS, bool BGK, bool LEAN>
+template <typename T, int BX, int BY, int BZ, bool WALLS, bool BGK>
 __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
                                   (BoxShape<BX, BY, BZ>::kCtasPerSm))
     k_fused_box(const T* __restrict__ src, T* __restrict__ dst,
@@ -118,11 +118,11 @@ __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
       [&](int dx, int dy, int dz) -> const float4& { return win[sz + dz][sy + dy][sx + dx]; },
       ctr, xlo, xhi, ylo, yhi, zlo, zhi, Gx, Gy, Gz, Qx, Qy, Qz);
   if (WALLS && a.wetting) wetting_rule(a, xlo, xhi, ylo, yhi, zlo, zhi, Gx, Gy, Gz);
-  const auto rc = collide_as<LEAN, BGK>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+  const auto rc = collide_stored<T, BGK>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
   store_recoloured<T>(dst, (unsigned)a.plane, a, cell, rc, f);
 }
 
-template <typename T, int BX, int BY, int BZ, bool WALLS, bool BGK, bool LEAN>
+template <typename T, int BX, int BY, int BZ, bool WALLS, bool BGK>
 static cudaError_t launch_box_v(const void* src, void* dst, const StepArgs& a, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY, (a.nz + BZ - 1) / BZ);
@@ -133,29 +133,25 @@ static cudaError_t launch_box_v(const void* src, void* dst, const StepArgs& a, c
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_fused_box<T, BX, BY, BZ, WALLS, BGK, LEAN>, (const T*)src,
-                            (T*)dst, a);
+  return cudaLaunchKernelEx(&cfg, k_fused_box<T, BX, BY, BZ, WALLS, BGK>, (const T*)src, (T*)dst,
+                            a);
 }
 
-template <typename T, int BX, int BY, int BZ, bool BGK>
+template <typename T, int BX, int BY, int BZ>
 static cudaError_t launch_box_b(const void* src, void* dst, const StepArgs& a, cudaStream_t s) {
-  if (!(a.wx || a.wy || a.wz)) return launch_box_v<T, BX, BY, BZ, false, BGK, true>(src, dst, a, s);
-  if (lean_collision<T>(a)) return launch_box_v<T, BX, BY, BZ, true, BGK, true>(src, dst, a, s);
-  if constexpr (!Store<T>::kDeviation)
-    return launch_box_v<T, BX, BY, BZ, true, BGK, false>(src, dst, a, s);
-  return cudaErrorInvalidValue;
+  if (a.wx || a.wy || a.wz)
+    return a.bgk ? launch_box_v<T, BX, BY, BZ, true, true>(src, dst, a, s)
+                 : launch_box_v<T, BX, BY, BZ, true, false>(src, dst, a, s);
+  return a.bgk ? launch_box_v<T, BX, BY, BZ, false, true>(src, dst, a, s)
+               : launch_box_v<T, BX, BY, BZ, false, false>(src, dst, a, s);
 }
 
 template <typename T>
 cudaError_t launch_fused_box_storage(const void* src, void* dst, const StepArgs& a, int box,
                                      cudaStream_t s) {
   switch (box) {
-    case 1:
-      return a.bgk ? launch_box_b<T, 4, 4, 4, true>(src, dst, a, s)
-                   : launch_box_b<T, 4, 4, 4, false>(src, dst, a, s);
-    case 2:
-      return a.bgk ? launch_box_b<T, 8, 4, 4, true>(src, dst, a, s)
-                   : launch_box_b<T, 8, 4, 4, false>(src, dst, a, s);
+    case 1: return launch_box_b<T, 4, 4, 4>(src, dst, a, s);
+    case 2: return launch_box_b<T, 8, 4, 4>(src, dst, a, s);
   }
   return cudaErrorInvalidValue;
 }

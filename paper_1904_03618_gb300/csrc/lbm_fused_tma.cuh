@@ -661,7 +661,7 @@ __device__ __forceinline__ void monitor_flush(const MonSlot* slots, MonAcc* g, i
 // seam only; its lanes whose sources lie beyond the high seam pull from
 // global memory.
 template <typename T, bool WALLS, int TW, int BY, int NS, bool SEAM = false,
-          bool FALLBACK = false, bool MON = false, bool LEAN = Store<T>::kDeviation>
+          bool FALLBACK = false, bool MON = false>
 __device__ __forceinline__ bool tma_chunk(const T* __restrict__ src, T* __restrict__ dst,
                                           const StepArgs& a, const CUtensorMap* map0,
                                           const CUtensorMap* map1, int bx, int by, int zb,
@@ -913,7 +913,7 @@ __device__ __forceinline__ bool tma_chunk(const T* __restrict__ src, T* __restri
       const Macro m = HV == 24 ? macro_held(a, ch[0], ch[1], ch[2], ch[3], ch[4])
                                : macro_total(a, cf, ch[0], ch[1]);
       if constexpr (MON) monitor_lane_add(ml, m, ctr.x, z);
-      const auto rc = collide_as<LEAN>(a, cf, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+      const auto rc = collide_stored<T>(a, cf, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
       store_recoloured<T>(dst, plane, a, (unsigned)z * g.plane_cells + g.co.yo[1] + g.co.xo[1],
                           rc, cf);
       get(cf, ch);
@@ -940,7 +940,7 @@ __device__ __forceinline__ unsigned char* tma_mbar_bytes(unsigned char* smem) {
          tma_hold_bytes<TW, BY>(tma_hold_vals<T, TW, BY, NS, SEAM>());
 }
 
-template <typename T, bool WALLS, int TW, int BY, int NS, bool LEAN>
+template <typename T, bool WALLS, int TW, int BY, int NS>
 __global__ void __launch_bounds__(TW* BY, (tma_ctas_per_sm<TW, BY>()))
     k_fused_tma(const T* __restrict__ src, T* __restrict__ dst,
                 const __grid_constant__ StepArgs a, const __grid_constant__ CUtensorMap map0,
@@ -955,8 +955,8 @@ __global__ void __launch_bounds__(TW* BY, (tma_ctas_per_sm<TW, BY>()))
   }
   tma_init_barriers(tma_mbar_bytes<T, TW, BY, NS>(smem), NS);
   __syncthreads();
-  tma_chunk<T, WALLS, TW, BY, NS, false, false, false, LEAN>(
-      src, dst, a, &map0, &map1, blockIdx.x, blockIdx.y, zb, ze, smem, 0u, err, tma_wait_limit());
+  tma_chunk<T, WALLS, TW, BY, NS>(src, dst, a, &map0, &map1, blockIdx.x, blockIdx.y, zb, ze,
+                                  smem, 0u, err, tma_wait_limit());
 }
 
 // SEAM form (FP32, periodic in x and y, one stage): the source buffer's six
@@ -993,7 +993,7 @@ __global__ void __launch_bounds__(TW* BY, 1)
   tma_init_barriers(tma_mbar_bytes<float, TW, BY, NS, true>(smem), NS);
   __syncthreads();
   const SeamStripMaps strips = {&mxs, &mys0, &mys1, &mcs};
-  const bool ok = tma_chunk<float, WALLS, TW, BY, NS, true, false, MON, true>(
+  const bool ok = tma_chunk<float, WALLS, TW, BY, NS, true, false, MON>(
       src, dst, a, &map0, &map1, blockIdx.x, blockIdx.y, zb, ze, smem, 0u, err,
       tma_wait_limit(), &strips, macc);
   if constexpr (MON) {
@@ -1246,8 +1246,8 @@ static cudaError_t launch_tma_seam_batch_v(const void* src, void* dst, const Bat
 
 // Tensor maps are built on the host (lbm_dispatch.cu); the launcher only
 // sets the dynamic shared-memory limit once per instantiation.
-template <typename T, bool WALLS, int TW, int BY, int NS, bool LEAN>
-static cudaError_t launch_tma_l(const void* src, void* dst, const StepArgs& a,
+template <typename T, bool WALLS, int TW, int BY, int NS>
+static cudaError_t launch_tma_v(const void* src, void* dst, const StepArgs& a,
                                 const CUtensorMap* maps, int zc, int* err, cudaStream_t s) {
   if constexpr (!tma_fits<T, TW, BY, NS>()) {
     return cudaErrorInvalidValue;
@@ -1256,26 +1256,17 @@ static cudaError_t launch_tma_l(const void* src, void* dst, const StepArgs& a,
     const int dv = device_slot();
     constexpr int bytes = tma_smem_bytes<T, TW, BY, NS>();
     if (!attr_set[dv]) {
-      cudaError_t e = cudaFuncSetAttribute(k_fused_tma<T, WALLS, TW, BY, NS, LEAN>,
+      cudaError_t e = cudaFuncSetAttribute(k_fused_tma<T, WALLS, TW, BY, NS>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
       if (e != cudaSuccess) return e;
       attr_set[dv] = true;
     }
     dim3 blk(TW, BY);
     dim3 grd((a.nx + TW - 3) / (TW - 2), (a.ny + BY - 3) / (BY - 2), (a.nz + zc - 1) / zc);
-    k_fused_tma<T, WALLS, TW, BY, NS, LEAN>
-        <<<grd, blk, bytes, s>>>((const T*)src, (T*)dst, a, maps[0], maps[1], zc, err);
+    k_fused_tma<T, WALLS, TW, BY, NS><<<grd, blk, bytes, s>>>((const T*)src, (T*)dst, a, maps[0],
+                                                             maps[1], zc, err);
     return cudaGetLastError();
   }
-}
-
-template <typename T, bool WALLS, int TW, int BY, int NS>
-static cudaError_t launch_tma_v(const void* src, void* dst, const StepArgs& a,
-                                const CUtensorMap* maps, int zc, int* err, cudaStream_t s) {
-  if constexpr (WALLS && !Store<T>::kDeviation)
-    if (!lean_collision<T>(a))
-      return launch_tma_l<T, WALLS, TW, BY, NS, false>(src, dst, a, maps, zc, err, s);
-  return launch_tma_l<T, WALLS, TW, BY, NS, true>(src, dst, a, maps, zc, err, s);
 }
 
 template <typename T, bool WALLS>
