@@ -622,229 +622,9 @@ __device__ __forceinline__ Recolour collide_total(const StepArgs& a, float* f,
   return rc;
 }
 
-// ---------------------------------------------------------------------------
-// The same collision with fewer operations (about a tenth of the step's): the
-// residuals m^eq - m from shared products (rho u_a u_b, A = rho |u|^2), sources
-// only where there are any, recolouring terms formed once per axis.  Its
-// results differ from collide_total's in the last bits, so it runs where nothing
-// is held to those bits: in 16-bit storage, whose stores round 10^4 times more
-// coarsely, and in the in-place step.  (FP32 steps keep collide_total's bits:
-// drops at relaxation times near 1/2 multiply a changed last bit a thousandfold
-// within 24 steps.)  GB300, us per step: 192 x 192 x 768 BF16 1553 -> 1500, FP16
-// droplet sweep 1189 -> 1150, 128^3 FP16 121.1 -> 120.0, in place 192 x 192 x 768
-// FP32 2675 -> 2641.
-// ---------------------------------------------------------------------------
-struct RecolourLean {
-  float wr, wb;
-  float nx, ny, nz, cax;  // axis terms cax n (n any multiple of the direction)
-  float dx, dy, dz;       // diagonal terms, summed over the axes
-};
-
-template <int I>
-__device__ __forceinline__ float recolour_seg(const RecolourLean& rc) {
-  if (I == 0) return 0.f;
-  if (shell(I) == 1) return rc.cax * (ex(I) * rc.nx + ey(I) * rc.ny + ez(I) * rc.nz);
-  return ex(I) * rc.dx + ey(I) * rc.dy + ez(I) * rc.dz;
-}
-
-struct Residual {
-  float r[19];  // m^eq - m, rows 4..18 (the others unused)
-};
-
-__device__ __forceinline__ float pressure(const StepArgs& a, const Macro& mc) {
-  return a.cs2_R * mc.rR + a.cs2_B * mc.rB;  // sum_k rho_k (c_s^k)^2
-}
-
-__device__ __forceinline__ Residual collide_pre(const StepArgs& a, const float* f,
-                                                const Macro& mc) {
-  Residual R;
-  const float ux = mc.ux, uy = mc.uy, uz = mc.uz;
-  // equilibria summed over colours, from rho u_a u_b (A the sum of the squares)
-  const float p = pressure(a, mc);
-  const float pc = a.improved ? p : mc.rho * (1.0f / 3.0f);
-  const float rx = mc.rho * ux, ry = mc.rho * uy, rz = mc.rho * uz;
-  const float xx = rx * ux, yy = ry * uy, zz = rz * uz;
-  const float A = xx + yy + zz;
-  const float t = (p + A) * (1.0f / 3.0f);
-  // raw moments of Eq. 43, rows 4..18, by opposite pairs
-  const float a12 = f[1] + f[2], a34 = f[3] + f[4], a56 = f[5] + f[6];
-  const float p78 = f[7] + f[8], p90 = f[9] + f[10];
-  const float p12 = f[11] + f[12], p34 = f[13] + f[14];
-  const float p56 = f[15] + f[16], p78b = f[17] + f[18];
-  const float Sxy = p78 + p90, Sxz = p12 + p34, Syz = p56 + p78b;
-  const float ax = a12 + a34 + a56, dg = Sxy + Sxz + Syz;
-  R.r[4] = (3.f * p + A) - (ax + 2.f * dg);
-  R.r[5] = (3.f * xx - A) - (3.f * (a12 - Syz) + (dg - ax));
-  R.r[6] = (yy - zz) - ((a34 - a56) + (Sxy - Sxz));
-  R.r[7] = rx * uy - (p78 - p90);
-  R.r[8] = rx * uz - (p12 - p34);
-  R.r[9] = ry * uz - (p56 - p78b);
-  const float d78 = f[7] - f[8], d90 = f[9] - f[10];
-  const float d12 = f[11] - f[12], d34 = f[13] - f[14];
-  const float d56 = f[15] - f[16], d78b = f[17] - f[18];
-  R.r[10] = pc * uy - (d78 - d90);
-  R.r[11] = pc * ux - (d78 + d90);
-  R.r[12] = pc * uz - (d12 - d34);
-  R.r[13] = pc * ux - (d12 + d34);
-  R.r[14] = pc * uz - (d56 - d78b);
-  R.r[15] = pc * uy - (d56 + d78b);
-  R.r[16] = (t - 0.5f * zz) - Sxy;
-  R.r[17] = (t - 0.5f * yy) - Sxz;
-  R.r[18] = (t - 0.5f * xx) - Syz;
-  return R;
-}
-
-// BGK: the operator of Eq. 20 (Lambda = I / tau_v), a compile-time choice:
-// in the MRT form the rates of rows 4 and 10-18 are launch constants, so
-// their relaxation does not wait for tau_v.
-template <bool BGK = false>
-__device__ __forceinline__ RecolourLean collide_post(const StepArgs& a, float* f, const Residual& R,
-                                                 const Macro& mc, float rhoN, float Gx, float Gy,
-                                                 float Gz, float Qx, float Qy, float Qz) {
-  const float Fx = mc.Fx, Fy = mc.Fy, Fz = mc.Fz;
-
-  // perturbation moments (A/2)|G| pi(n), pi from M applied to Eq. 8; without a
-  // gradient (or with a NaN in it) no perturbation and no recolouring direction
-  if (!(Gx * Gx + Gy * Gy + Gz * Gz >= 1e-24f)) Gx = Gy = Gz = 0.f;
-  const float xx = Gx * Gx, yy = Gy * Gy, zz = Gz * Gz;
-  const float G2 = xx + yy + zz;
-  const float ig = G2 > 0.f ? rsqrtf(G2) : 0.f;
-  const float k19 = a.half_A * ig * (1.0f / 9.0f), k29 = 2.f * k19;
-  const float kx = k29 * Gx;
-
-  // relaxation rates (Eq. 44) with the variable tau_v of Eq. 52; the BGK
-  // operator of Eq. 20 is Lambda = I / tau_v, every rate 1 / tau_v (the
-  // conserved rows carry only F, whatever their rate)
-  const float s_v = fast_rcp(tau_v_of(a, rhoN));
-  const float s_e = BGK ? s_v : a.s_e;
-  const float s_q = BGK ? s_v : a.s_q;
-  const float s_pi = BGK ? s_v : a.s_pi;
-
-  // change of moments dm = m* - m (rows 1-3: F; row 0: 0)
-  float d[19];
-  d[4] = s_e * (R.r[4] - 4.f * k19 * G2);
-  d[5] = s_v * (R.r[5] + k29 * (3.f * xx - G2));
-  d[6] = s_v * (R.r[6] + k29 * (yy - zz));
-  d[7] = s_v * (R.r[7] + kx * Gy);
-  d[8] = s_v * (R.r[8] + kx * Gz);
-  d[9] = s_v * (R.r[9] + k29 * Gy * Gz);
-#pragma unroll
-  for (int r = 10; r <= 15; ++r) d[r] = s_q * R.r[r];
-  d[16] = s_pi * (R.r[16] - k19 * zz);
-  d[17] = s_pi * (R.r[17] - k19 * yy);
-  d[18] = s_pi * (R.r[18] - k19 * xx);
-  // source in moment space under (1 - s / 2): correction C (rows 4-6) ...
-  const float g_e = 1.f - 0.5f * s_e, g_v = 1.f - 0.5f * s_v;
-  if (a.improved) {
-    const float Q = Qx + Qy + Qz;
-    d[4] += g_e * Q;
-    d[5] += g_v * (3.f * Qx - Q);
-    d[6] += g_v * (Qy - Qz);
-  }
-  // ... and the Guo force F_hat
-  d[1] = d[2] = d[3] = 0.f;
-  if (a.has_force) {
-    const float ux = mc.ux, uy = mc.uy, uz = mc.uz;
-    const float fx = Fx * ux, fy = Fy * uy, fz = Fz * uz, fs = fx + fy + fz;
-    const float g_q = (1.f - 0.5f * s_q) * (1.0f / 3.0f), g_pi = 1.f - 0.5f * s_pi;
-    d[1] = Fx;
-    d[2] = Fy;
-    d[3] = Fz;
-    d[4] += g_e * (2.f * fs);
-    d[5] += g_v * (6.f * fx - 2.f * fs);
-    d[6] += g_v * (2.f * (fy - fz));
-    d[7] += g_v * (Fx * uy + Fy * ux);
-    d[8] += g_v * (Fx * uz + Fz * ux);
-    d[9] += g_v * (Fy * uz + Fz * uy);
-    d[10] += g_q * Fy;
-    d[11] += g_q * Fx;
-    d[12] += g_q * Fz;
-    d[13] += g_q * Fx;
-    d[14] += g_q * Fz;
-    d[15] += g_q * Fy;
-    const float t = (2.0f / 3.0f) * fs;
-    d[16] += g_pi * (t - fz);
-    d[17] += g_pi * (t - fy);
-    d[18] += g_pi * (t - fx);
-  }
-
-  // f* = f + M^-1 dm (sparse closed form of the inverse of Eq. 43)
-  const float h = 0.5f, q = 0.25f;
-  const float s67 = d[16] + d[17];
-  f[0] += (s67 + d[18]) - d[4];
-  const float c4 = d[4] * (1.0f / 6.0f), c5 = d[5] * (1.0f / 12.0f);
-  {
-    const float base = c4 + 2.f * c5 - h * s67;
-    const float odd = h * (d[1] - (d[11] + d[13]));
-    f[1] += base + odd;
-    f[2] += base - odd;
-  }
-  const float c45 = c4 - c5;
-  {
-    const float base = c45 + q * d[6] - h * (d[16] + d[18]);
-    const float odd = h * (d[2] - (d[10] + d[15]));
-    f[3] += base + odd;
-    f[4] += base - odd;
-  }
-  {
-    const float base = c45 - q * d[6] - h * (d[17] + d[18]);
-    const float odd = h * (d[3] - (d[12] + d[14]));
-    f[5] += base + odd;
-    f[6] += base - odd;
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    // directions i .. i + 3 of a diagonal plane: even moments d[16 + k], d[7 +
-    // k], odd ones d[10 + 2 k], d[11 + 2 k]
-    const int i = 7 + 4 * k;
-    const float sp = d[16 + k] + d[7 + k], sm = d[16 + k] - d[7 + k];
-    const float op = d[11 + 2 * k] + d[10 + 2 * k], om = d[11 + 2 * k] - d[10 + 2 * k];
-    f[i] += q * (sp + op);
-    f[i + 1] += q * (sp - op);
-    f[i + 2] += q * (sm + om);
-    f[i + 3] += q * (sm - om);
-  }
-
-  RecolourLean rc;
-  rc.wr = mc.rR * mc.inv_rho;
-  rc.wb = mc.rB * mc.inv_rho;
-  // seg_i = c_shell(i) (e_i . n), zero without a gradient
-  const float cb = a.beta * rc.wr * rc.wb * pressure(a, mc) * ig;
-  rc.cax = cb * (1.0f / 6.0f);
-  const float cdg = cb * (1.0f / (12.0f * 1.41421356237309515f));
-  rc.nx = Gx;
-  rc.ny = Gy;
-  rc.nz = Gz;
-  rc.dx = cdg * Gx;
-  rc.dy = cdg * Gy;
-  rc.dz = cdg * Gz;
-  return rc;
-}
-
-
-template <bool BGK = false>
-__device__ __forceinline__ RecolourLean collide_lean(const StepArgs& a, float* f, const Macro& mc,
-                                                     float rhoN, float Gx, float Gy, float Gz,
-                                                     float Qx, float Qy, float Qz) {
-  const Residual R = collide_pre(a, f, mc);
-  return collide_post<BGK>(a, f, R, mc, rhoN, Gx, Gy, Gz, Qx, Qy, Qz);
-}
-
-// The collision a kernel of storage type T runs.
-template <typename T, bool BGK = false>
-__device__ __forceinline__ auto collide_stored(const StepArgs& a, float* f, const Macro& mc,
-                                               float rhoN, float Gx, float Gy, float Gz, float Qx,
-                                               float Qy, float Qz) {
-  if constexpr (Store<T>::kDeviation)
-    return collide_lean<BGK>(a, f, mc, rhoN, Gx, Gy, Gz, Qx, Qy, Qz);
-  else
-    return collide_total<BGK>(a, f, mc, rhoN, Gx, Gy, Gz, Qx, Qy, Qz);
-}
-
 template <int I>
 struct RecolourAll {
-  template <typename Rc>
-  __device__ __forceinline__ static void run(const Rc& rc,
+  __device__ __forceinline__ static void run(const Recolour& rc,
                                              const float* fs, float* fR,
                                              float* fB) {
     const float sg = recolour_seg<I>(rc);
@@ -855,8 +635,7 @@ struct RecolourAll {
 };
 template <>
 struct RecolourAll<19> {
-  template <typename Rc>
-  __device__ __forceinline__ static void run(const Rc&, const float*,
+  __device__ __forceinline__ static void run(const Recolour&, const float*,
                                              float*, float*) {}
 };
 

@@ -118,7 +118,7 @@ __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
       [&](int dx, int dy, int dz) -> const float4& { return win[sz + dz][sy + dy][sx + dx]; },
       ctr, xlo, xhi, ylo, yhi, zlo, zhi, Gx, Gy, Gz, Qx, Qy, Qz);
   if (WALLS && a.wetting) wetting_rule(a, xlo, xhi, ylo, yhi, zlo, zhi, Gx, Gy, Gz);
-  const auto rc = collide_stored<T, BGK>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+  const Recolour rc = collide_total<BGK>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
   store_recoloured<T>(dst, (unsigned)a.plane, a, cell, rc, f);
 }
 

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kInplaceBlock, 4)
     wetting_rule(a, a.wx && s.x == 0, a.wx && s.x == a.nx - 1, a.wy && s.y == 0,
                  a.wy && s.y == a.ny - 1, a.wz && s.z == 0, a.wz && s.z == a.nz - 1, Gx, Gy,
                  Gz);
-  const RecolourLean rc = collide_lean<BGK>(a, ft, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+  const Recolour rc = collide_total<BGK>(a, ft, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
   float fR[19], fB[19];
   RecolourAll<0>::run(rc, ft, fR, fB);
   n.refresh();
