@@ -23,6 +23,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lbm_chained.cuh"
+
 namespace lbm {
 
 // ---------------------------------------------------------------------------

@@ -48,8 +48,9 @@ __device__ __forceinline__ void add_offsets(const StepArgs& a, float2& v) {
 // Pull of the 19 pairs of one column / plane, reduced on the fly to
 // (f_i = fR_i + fB_i, rho_R, rho_B).  The colour sums run as one paired
 // FP32 add per direction (the red and blue values arrive as a pair; each
-// component rounds as its scalar add would).
-template <typename T, bool WALLS, int I>
+// component rounds as its scalar add would).  CHAINED: src is written while the
+// kernel waits to start (ld_chained).
+template <typename T, bool WALLS, int I, bool CHAINED>
 struct PullReduce {
   __device__ __forceinline__ static void run(const typename Store<T>::Pair* src,
                                              unsigned plane, const StepArgs& a,
@@ -57,27 +58,30 @@ struct PullReduce {
                                              float* f, float2& rho) {
     const unsigned q = pull_index<WALLS, I>(plane, c, p);
     float2 v = make_float2(0.f, 0.f);
-    if (index_ok(a, q, 19ull * plane)) v = Store<T>::to_float2(__ldg(src + q));
+    if (index_ok(a, q, 19ull * plane)) {
+      if constexpr (CHAINED) v = Store<T>::to_float2(ld_chained(src + q));
+      else v = Store<T>::to_float2(__ldg(src + q));
+    }
     add_offsets<T, I>(a, v);
     rho = __fadd2_rn(rho, v);
     f[I] = v.x + v.y;
-    PullReduce<T, WALLS, I + 1>::run(src, plane, a, c, p, f, rho);
+    PullReduce<T, WALLS, I + 1, CHAINED>::run(src, plane, a, c, p, f, rho);
   }
 };
-template <typename T, bool WALLS>
-struct PullReduce<T, WALLS, 19> {
+template <typename T, bool WALLS, bool CHAINED>
+struct PullReduce<T, WALLS, 19, CHAINED> {
   __device__ __forceinline__ static void run(const typename Store<T>::Pair*,
                                              unsigned, const StepArgs&,
                                              const ColOff&, const PlaneOff&,
                                              float*, float2&) {}
 };
-template <typename T, bool WALLS>
+template <typename T, bool WALLS, bool CHAINED = false>
 __device__ __forceinline__ void pull_reduce(const typename Store<T>::Pair* src, unsigned plane,
                                             const StepArgs& a, const ColOff& c,
                                             const PlaneOff& p, float* f, float& rR,
                                             float& rB) {
   float2 rho = make_float2(rR, rB);
-  PullReduce<T, WALLS, 0>::run(src, plane, a, c, p, f, rho);
+  PullReduce<T, WALLS, 0, CHAINED>::run(src, plane, a, c, p, f, rho);
   rR = rho.x;
   rB = rho.y;
 }

@@ -69,8 +69,7 @@ struct BoxShape {
 template <typename T, int BX, int BY, int BZ, bool WALLS, bool BGK>
 __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
                                   (BoxShape<BX, BY, BZ>::kCtasPerSm))
-    k_fused_box(const T* __restrict__ src, T* __restrict__ dst,
-                const __grid_constant__ StepArgs a) {
+    k_fused_box(const T* src, T* dst, const __grid_constant__ StepArgs a) {
   using S = BoxShape<BX, BY, BZ>;
   using Pair = typename Store<T>::Pair;
   __shared__ float4 win[S::SZ][S::SY][S::SX];
@@ -78,10 +77,8 @@ __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
   int sx, sy, sz;
   S::site(t, sx, sy, sz);
   // launched with programmatic stream serialisation: the next step's CTAs may
-  // start (and wait here) while this one runs, which hides their launch; the
-  // wait returns once the step before has completed and its stores are visible
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  // start (and wait here) while this one runs, which hides their launch
+  after_previous_kernel();
   const int cx = blockIdx.x * BX + sx - 1, cy = blockIdx.y * BY + sy - 1,
             cz = blockIdx.z * BZ + sz - 1;  // unwrapped
   // sites that some cell of the box reads: inside the lattice or one cell
@@ -102,8 +99,8 @@ __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
     const ColOff co = col_off(a, x, y);
     const PlaneOff po = plane_off(a, z);
     cell = po.zo[1] + co.yo[1] + co.xo[1];
-    pull_reduce<T, WALLS>(reinterpret_cast<const Pair*>(src), (unsigned)a.plane, a, co, po, f, rR,
-                          rB);
+    pull_reduce<T, WALLS, true>(reinterpret_cast<const Pair*>(src), (unsigned)a.plane, a, co, po,
+                                f, rR, rB);
     m = macro_total(a, f, rR, rB);
     win[sz][sy][sx] = stencil_entry(a, m);
   }

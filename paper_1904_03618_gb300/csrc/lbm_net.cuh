@@ -34,6 +34,8 @@
 // A training step of 256 rows: 37 us against 226 us.
 #pragma once
 
+#include "lbm_chained.cuh"
+
 namespace lbm {
 namespace mlp {
 
@@ -235,7 +237,7 @@ __device__ __forceinline__ void net_input_tile(const NetArgs& g, unsigned char* 
     float v[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j)
-      v[j] = m < g.batch && k + j < n_in ? __ldg(g.x + (size_t)m * n_in + k + j) : 0.f;
+      v[j] = m < g.batch && k + j < n_in ? ld_chained(g.x + (size_t)m * n_in + k + j) : 0.f;
     *reinterpret_cast<uint4*>(act + act_offset(r, k)) = pack8(v);
   }
 }
@@ -436,12 +438,7 @@ __global__ void __launch_bounds__(kNetThreads, 1)
 }
 
 // The kernels of a training step are launched with programmatic stream
-// serialisation: each may start while the one before still runs and waits
-// here, before it touches memory, until that one has completed.
-__device__ __forceinline__ void after_previous_kernel() {
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
+// serialisation; what one writes, the next reads with ld_chained.
 
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
@@ -583,7 +580,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_net_cluster(const __grid_cons
           }
         } else {
           const int n = c + (lane & 15);
-          if (n < N) bias = __ldg(g.theta + s.woff(l) + (long long)s.din(l) * N + n);
+          if (n < N) bias = ld_chained(g.theta + s.woff(l) + (long long)s.din(l) * N + n);
         }
         ok = __all_sync(0xffffffffu, ws_wait(smem_u32(&sm.acc_full), q & 1, wait_ns, give_up));
         if (ok) {
@@ -622,7 +619,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_net_cluster(const __grid_cons
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
                 const float d =
-                    live && c + i < N ? v[i] - __ldg(g.t + (size_t)m * N + c + i) : 0.f;
+                    live && c + i < N ? v[i] - ld_chained(g.t + (size_t)m * N + c + i) : 0.f;
                 v[i] = 2.f * d * g.scale;
                 loss += d * d;
               }
@@ -723,7 +720,7 @@ __device__ __forceinline__ void dw_bias(float (*buf)[kDwK][kDwN], const float* Z
 #pragma unroll
     for (int i = 0; i < R; ++i) {
       const int k = k0 + p + i * P;
-      v[i] = k < batch && n0 + c < dout ? __ldg(Z + (size_t)k * dout + n0 + c) : 0.f;
+      v[i] = k < batch && n0 + c < dout ? ld_chained(Z + (size_t)k * dout + n0 + c) : 0.f;
     }
   };
   load(0);
@@ -744,7 +741,7 @@ __device__ __forceinline__ void dw_bias(float (*buf)[kDwK][kDwN], const float* Z
 // the core layout, zero outside R x K.  A task is 4 rows x 8 k: eight 16-byte
 // loads along the rows, transposed in registers into four 16-byte stores.
 template <int ROWS>
-__device__ __forceinline__ void dw_stage(unsigned char* dst, const float* __restrict__ src, int ld,
+__device__ __forceinline__ void dw_stage(unsigned char* dst, const float* src, int ld,
                                          int r0, int R, int K, int t) {
   constexpr int quads = ROWS / 4, G = quads * (kDwK / 8);
   const bool vec = (ld & 3) == 0 && ((size_t)src & 15u) == 0;
@@ -758,12 +755,12 @@ __device__ __forceinline__ void dw_stage(unsigned char* dst, const float* __rest
       if (k + j >= K || m >= R) continue;
       const float* p = src + (size_t)(k + j) * ld + m;
       if (vec && m + 3 < R) {
-        v[j] = __ldg(reinterpret_cast<const float4*>(p));
+        v[j] = ld_chained(reinterpret_cast<const float4*>(p));
       } else {
-        v[j].x = __ldg(p);
-        if (m + 1 < R) v[j].y = __ldg(p + 1);
-        if (m + 2 < R) v[j].z = __ldg(p + 2);
-        if (m + 3 < R) v[j].w = __ldg(p + 3);
+        v[j].x = ld_chained(p);
+        if (m + 1 < R) v[j].y = ld_chained(p + 1);
+        if (m + 2 < R) v[j].z = ld_chained(p + 2);
+        if (m + 3 < R) v[j].w = ld_chained(p + 3);
       }
     }
     const float* f = reinterpret_cast<const float*>(v);
@@ -893,15 +890,13 @@ __global__ void k_net_pack(const __grid_constant__ NetShape s, const float* __re
 
 // One Adam step over all parameters (bias-corrected, Kingma & Ba); the
 // updated weights also go into the packed copies.
-__global__ void k_net_adam(const __grid_constant__ NetShape s, float* __restrict__ p,
-                           const float* __restrict__ g, float* __restrict__ m,
-                           float* __restrict__ v, long long n, float lr, float b1, float b2,
-                           float eps, float c1, float c2, __nv_bfloat16* __restrict__ fwd,
-                           __nv_bfloat16* __restrict__ bwd) {
+__global__ void k_net_adam(const __grid_constant__ NetShape s, float* p, const float* g, float* m,
+                           float* v, long long n, float lr, float b1, float b2, float eps,
+                           float c1, float c2, __nv_bfloat16* fwd, __nv_bfloat16* bwd) {
   after_previous_kernel();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float gi = g[i];
+  const float gi = ld_chained(g + i);
   const float mi = b1 * m[i] + (1.f - b1) * gi;
   const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
   m[i] = mi;
