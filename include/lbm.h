@@ -297,7 +297,7 @@ lbm_status lbm_set_planes(lbm_ctx *ctx, int z0, int n, const void *src);
    (interior 32 x 10) with two stages, accepted only there and the default
    there.  The TMA waits are bounded and report LBM_ERR_TIMEOUT through
    lbm_diagnostics.
-   Small single lattices (up to 81,920 cells where a seam form exists,
+   Small single MRT lattices (up to 81,920 cells where a seam form exists,
    180,000 elsewhere) step by default in a form of their own, one CTA per
    box of 4 x 4 x 4 or 8 x 4 x 4 cells, whatever the configuration
    lbm_create reports; a configuration set here runs the kernel it names,

@@ -66,7 +66,7 @@ struct BoxShape {
   }
 };
 
-template <typename T, int BX, int BY, int BZ, bool WALLS, bool BGK>
+template <typename T, int BX, int BY, int BZ, bool WALLS>
 __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
                                   (BoxShape<BX, BY, BZ>::kCtasPerSm))
     k_fused_box(const T* src, T* dst, const __grid_constant__ StepArgs a) {
@@ -115,11 +115,11 @@ __global__ void __launch_bounds__((BoxShape<BX, BY, BZ>::kThreads),
       [&](int dx, int dy, int dz) -> const float4& { return win[sz + dz][sy + dy][sx + dx]; },
       ctr, xlo, xhi, ylo, yhi, zlo, zhi, Gx, Gy, Gz, Qx, Qy, Qz);
   if (WALLS && a.wetting) wetting_rule(a, xlo, xhi, ylo, yhi, zlo, zhi, Gx, Gy, Gz);
-  const Recolour rc = collide_total<BGK>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+  const Recolour rc = collide_total<false>(a, f, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
   store_recoloured<T>(dst, (unsigned)a.plane, a, cell, rc, f);
 }
 
-template <typename T, int BX, int BY, int BZ, bool WALLS, bool BGK>
+template <typename T, int BX, int BY, int BZ, bool WALLS>
 static cudaError_t launch_box_v(const void* src, void* dst, const StepArgs& a, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((a.nx + BX - 1) / BX, (a.ny + BY - 1) / BY, (a.nz + BZ - 1) / BZ);
@@ -130,17 +130,13 @@ static cudaError_t launch_box_v(const void* src, void* dst, const StepArgs& a, c
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_fused_box<T, BX, BY, BZ, WALLS, BGK>, (const T*)src, (T*)dst,
-                            a);
+  return cudaLaunchKernelEx(&cfg, k_fused_box<T, BX, BY, BZ, WALLS>, (const T*)src, (T*)dst, a);
 }
 
 template <typename T, int BX, int BY, int BZ>
 static cudaError_t launch_box_b(const void* src, void* dst, const StepArgs& a, cudaStream_t s) {
-  if (a.wx || a.wy || a.wz)
-    return a.bgk ? launch_box_v<T, BX, BY, BZ, true, true>(src, dst, a, s)
-                 : launch_box_v<T, BX, BY, BZ, true, false>(src, dst, a, s);
-  return a.bgk ? launch_box_v<T, BX, BY, BZ, false, true>(src, dst, a, s)
-               : launch_box_v<T, BX, BY, BZ, false, false>(src, dst, a, s);
+  return a.wx || a.wy || a.wz ? launch_box_v<T, BX, BY, BZ, true>(src, dst, a, s)
+                              : launch_box_v<T, BX, BY, BZ, false>(src, dst, a, s);
 }
 
 template <typename T>

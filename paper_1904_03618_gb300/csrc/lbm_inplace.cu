@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kInplaceBlock)
 // 192-cell rows 8 %), 131^3 292 (232).  Tried on top and dropped: the phase
 // field of the next slab of planes in the launch of this slab's collision, to
 // find its populations in L2 (192 x 192 x 768 2890 at the best slab, 128^3 185).
-template <int ODD, bool BGK, typename Idx, bool WALLS, typename T>
+template <int ODD, typename Idx, bool WALLS, typename T>
 __global__ void __launch_bounds__(kInplaceBlock, 4)
     k_inplace_collide(T* f, StepArgs a, long long N, const float4* __restrict__ phase) {
   Site s;
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kInplaceBlock, 4)
     wetting_rule(a, a.wx && s.x == 0, a.wx && s.x == a.nx - 1, a.wy && s.y == 0,
                  a.wy && s.y == a.ny - 1, a.wz && s.z == 0, a.wz && s.z == a.nz - 1, Gx, Gy,
                  Gz);
-  const Recolour rc = collide_total<BGK>(a, ft, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+  const Recolour rc = collide_total<false>(a, ft, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
   float fR[19], fB[19];
   RecolourAll<0>::run(rc, ft, fR, fB);
   n.refresh();
@@ -325,6 +325,68 @@ __global__ void __launch_bounds__(kInplaceBlock, 4)
     const auto o = n.template slot<ODD>(opp(i));
     ip_store(f + o, fR[i], a, 0, i);
     ip_store(fb + o, fB[i], a, 1, i);
+  }
+}
+
+// Both passes of BGK lattices, with indices formed per thread and both colours
+// kept.  Every rate of that operator is 1 / tau_v, and near tau_v = 1/2 a changed
+// last bit grows until the fields are others: with the code above (whose
+// multiply-adds are contracted elsewhere) a closed box of drops is 4e-5 apart
+// after 60 steps and a Rayleigh-Taylor column overflows in other cells.  128^3
+// takes 217 us a step here.
+template <int ODD, typename T>
+__global__ void __launch_bounds__(kInplaceBlock)
+    k_inplace_phase_bgk(const T* __restrict__ f, StepArgs a, long long N,
+                    float4* __restrict__ phase) {
+  Site s;
+  if (!site_of(a, s)) return;
+  const Nbr nb = neighbourhood(a, s);
+  float fR[19], fB[19];
+  load_site<ODD>(f, a, nb, s, N, fR, fB);
+  phase[s.c] = stencil_entry(a, macro_of(a, fR, fB));
+}
+
+template <int ODD, typename T>
+__global__ void __launch_bounds__(kInplaceBlock, 4)
+    k_inplace_collide_bgk(T* f, StepArgs a, long long N, const float4* __restrict__ phase) {
+  Site s;
+  if (!site_of(a, s)) return;
+  const Nbr nb = neighbourhood(a, s);
+  float fR[19], fB[19];
+  load_site<ODD>(f, a, nb, s, N, fR, fB);
+  const Macro m = macro_of(a, fR, fB);
+  const float4 ctr = phase[s.c];
+  float Gx = 0.f, Gy = 0.f, Gz = 0.f, Qx = 0.f, Qy = 0.f, Qz = 0.f;
+#pragma unroll
+  for (int i = 1; i < 19; i += 2) {
+    const long long np = site_shift(nb, ex(i), ey(i), ez(i));
+    const long long nm = site_shift(nb, -ex(i), -ey(i), -ez(i));
+    const float4 vp = np < 0 ? ctr : phase[np];
+    const float4 vm = nm < 0 ? ctr : phase[nm];
+    const float w = (i <= 6) ? (1.0f / 6.0f) : (1.0f / 12.0f);
+    if (ex(i)) {
+      Gx += (ex(i) * w) * (vp.x - vm.x);
+      Qx += (ex(i) * w) * (vp.y - vm.y);
+    }
+    if (ey(i)) {
+      Gy += (ey(i) * w) * (vp.x - vm.x);
+      Qy += (ey(i) * w) * (vp.z - vm.z);
+    }
+    if (ez(i)) {
+      Gz += (ez(i) * w) * (vp.x - vm.x);
+      Qz += (ez(i) * w) * (vp.w - vm.w);
+    }
+  }
+  if (a.wetting)
+    wetting_rule(a, a.wx && s.x == 0, a.wx && s.x == a.nx - 1, a.wy && s.y == 0,
+                 a.wy && s.y == a.ny - 1, a.wz && s.z == 0, a.wz && s.z == a.nz - 1, Gx, Gy,
+                 Gz);
+  collide_cell<true>(a, fR, fB, m, ctr.x, Gx, Gy, Gz, Qx, Qy, Qz);
+#pragma unroll
+  for (int i = 0; i < 19; ++i) {
+    const long long o = slot_of<ODD>(nb, s, opp(i), N);
+    ip_store(f + o, fR[i], a, 0, i);
+    ip_store(f + 19 * N + o, fB[i], a, 1, i);
   }
 }
 
@@ -394,31 +456,34 @@ cudaError_t ip_set(const lbm_params* p, const StepArgs& a, long long N, void* f,
   k_inplace_set<T><<<site_grid(p), kInplaceBlock, 0, s>>>((T*)f, a, N, f_in);
   return cudaGetLastError();
 }
-template <int ODD, bool BGK, typename Idx, bool WALLS, typename T>
+template <int ODD, typename Idx, bool WALLS, typename T>
 void ip_passes(const StepArgs& a, long long N, T* f, float4* phase, cudaStream_t s) {
   const int t = block_threads(a.nx);
   const dim3 g((unsigned)((a.nx + t - 1) / t), (unsigned)a.ny, (unsigned)a.nz);
   k_inplace_phase<ODD, Idx, WALLS, T><<<g, t, 0, s>>>(f, a, N, phase);
-  k_inplace_collide<ODD, BGK, Idx, WALLS, T><<<g, t, 0, s>>>(f, a, N, phase);
+  k_inplace_collide<ODD, Idx, WALLS, T><<<g, t, 0, s>>>(f, a, N, phase);
 }
 
 template <int ODD, typename T>
-void ip_parity(const StepArgs& a, long long N, T* f, float4* phase, cudaStream_t s) {
-  using U64 = unsigned long long;
-  if (38 * N >= (1LL << 32))
-    a.bgk ? ip_passes<ODD, true, U64, true, T>(a, N, f, phase, s)
-          : ip_passes<ODD, false, U64, true, T>(a, N, f, phase, s);
-  else if (a.bgk) ip_passes<ODD, true, unsigned, true, T>(a, N, f, phase, s);
-  else if (a.wx || a.wy || a.wz) ip_passes<ODD, false, unsigned, true, T>(a, N, f, phase, s);
-  else ip_passes<ODD, false, unsigned, false, T>(a, N, f, phase, s);
+void ip_parity(const lbm_params* p, const StepArgs& a, long long N, T* f, float4* phase,
+               cudaStream_t s) {
+  if (a.bgk) {
+    k_inplace_phase_bgk<ODD, T><<<site_grid(p), kInplaceBlock, 0, s>>>(f, a, N, phase);
+    k_inplace_collide_bgk<ODD, T><<<site_grid(p), kInplaceBlock, 0, s>>>(f, a, N, phase);
+  } else if (38 * N >= (1LL << 32)) {
+    ip_passes<ODD, unsigned long long, true, T>(a, N, f, phase, s);
+  } else if (a.wx || a.wy || a.wz) {
+    ip_passes<ODD, unsigned, true, T>(a, N, f, phase, s);
+  } else {
+    ip_passes<ODD, unsigned, false, T>(a, N, f, phase, s);
+  }
 }
 
 template <typename T>
 cudaError_t ip_step(const lbm_params* p, const StepArgs& a, long long N, void* fv, int parity,
                     float4* phase, cudaStream_t s) {
-  (void)p;
-  if (parity) ip_parity<1, T>(a, N, (T*)fv, phase, s);
-  else ip_parity<0, T>(a, N, (T*)fv, phase, s);
+  if (parity) ip_parity<1, T>(p, a, N, (T*)fv, phase, s);
+  else ip_parity<0, T>(p, a, N, (T*)fv, phase, s);
   return cudaGetLastError();
 }
 template <typename T>
