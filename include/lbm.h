@@ -269,7 +269,10 @@ lbm_status lbm_get_planes(lbm_ctx *ctx, int z0, int n, void *dst);
 lbm_status lbm_set_planes(lbm_ctx *ctx, int z0, int n, const void *src);
 
 /* Launch configuration of the fused kernel (LBM_KERNEL_FUSED), the knob the
-   autotuner turns; results are identical for every valid configuration.
+   autotuner turns.  Every valid configuration runs the same arithmetic;
+   results agree to rounding -- the compiler contracts other multiply-add
+   pairs in other kernels; populations differ by at most 1e-6 of the largest
+   after three steps -- and do not depend on zchunk.
    Batch contexts accept (tile_y, hold) = (8, 2), (8, 0), (16, 1) and, when
    every case has an x row of 16-byte multiple length, the TMA forms (8 or
    15, 7 or 8); their default is then (15, 32, 8) for FP32 and (15, 32, 7)
@@ -297,15 +300,27 @@ lbm_status lbm_set_planes(lbm_ctx *ctx, int z0, int n, const void *src);
    (interior 32 x 10) with two stages, accepted only there and the default
    there.  The TMA waits are bounded and report LBM_ERR_TIMEOUT through
    lbm_diagnostics.
-   Small single MRT lattices (up to 81,920 cells where a seam form exists,
-   180,000 elsewhere) step by default in a form of their own, one CTA per
-   box of 4 x 4 x 4 or 8 x 4 x 4 cells, whatever the configuration
-   lbm_create reports; a configuration set here runs the kernel it names,
-   and setting the reported one again brings the box form back.
+   Small single MRT lattices step by default in a form of their own instead
+   (lbm_set_box below); a configuration set here always runs the kernel it
+   names.
    Errors: LBM_ERR_ARG. */
 lbm_status lbm_set_fused_config(lbm_ctx *ctx, int tile_y, int zchunk, int hold);
 lbm_status lbm_get_fused_config(const lbm_ctx *ctx, int *tile_y, int *zchunk,
                                 int *hold);
+
+/* The box form of the step of small single lattices: one CTA per box of 4 x
+   4 x 4 (box = 1) or 8 x 4 x 4 cells (2) in place of the kernel of the fused
+   configuration (0); results as for another configuration.  lbm_create picks
+   it for MRT lattices of up to 81,920 cells where a seam form exists and
+   180,000 elsewhere, lbm_default_box tells which (host only; 0 beyond).
+   lbm_get_box: the form lbm_step runs now.  lbm_set_box chooses it;
+   lbm_set_fused_config chooses 0.  lbm_step_monitored runs the kernel of the
+   configuration where that sums the diagnostics.
+   Errors: LBM_ERR_ARG (a box form for a batch, the two-pass kernel, the BGK
+   operator or ny or nz above 262,140; invalid parameters, NULL output). */
+lbm_status lbm_set_box(lbm_ctx *ctx, int box);
+int lbm_get_box(const lbm_ctx *ctx);
+lbm_status lbm_default_box(const lbm_params *p, int *box);
 
 /* The fused configuration lbm_create picks for a single lattice with these
    parameters on a GPU with `sms` streaming multiprocessors (0: 152, the

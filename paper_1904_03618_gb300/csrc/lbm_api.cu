@@ -28,9 +28,7 @@ struct lbm_ctx {
   int ncases;
   int storage, kernel;
   lbm::FusedConfig fused;
-  lbm::FusedConfig fused_default;  // the configuration create picked
-  int box_default;                 // ... and its box form (0: none), single lattices
-  int box;                         // box form in use: box_default while `fused` is the default
+  int box;                  // box form in use (0: the kernel of `fused`), single lattices
   cudaStream_t stream;
   int device, sms;
   size_t elem;              // bytes per stored population value
@@ -584,7 +582,7 @@ static lbm_status create_ctx(const lbm_params* ps, int ncases, void* cuda_stream
     }
   }
   if (st == LBM_OK && ncases == 1 && c->kernel == LBM_KERNEL_FUSED)
-    c->box_default = c->box = lbm::default_box(c->cases[0].args, c->storage);
+    c->box = lbm::default_box(c->cases[0].args, c->storage);
   if (st == LBM_OK && ncases > 1) {
     // tensor maps of every case for the batched TMA step (tile kinds 0, 2)
     bool all = true;
@@ -646,7 +644,6 @@ static lbm_status create_ctx(const lbm_params* ps, int ncases, void* cuda_stream
   if (st == LBM_OK && ncases > 1 &&
       lbm::dev_alloc((void**)&c->d_cases, sizeof(lbm::BatchCase) * ncases) != cudaSuccess)
     st = fail(nullptr, LBM_ERR_OOM, "cudaMalloc of the case table failed");
-  c->fused_default = c->fused;
   if (st == LBM_OK) {
     st = upload_case_table(c);
     if (st != LBM_OK) {
@@ -1300,13 +1297,39 @@ extern "C" lbm_status lbm_set_planes(lbm_ctx* c, int z0, int n, const void* src)
   return plane_copy(c, z0, n, const_cast<void*>(src), false);
 }
 
-// A configuration set explicitly runs the marching kernel it names; the one
-// that create picked brings back create's choice, the box form included.
+// A configuration set explicitly runs the marching kernel it names.
 static void use_config(lbm_ctx* c, const lbm::FusedConfig& f) {
-  const lbm::FusedConfig& d = c->fused_default;
   c->fused = f;
-  c->box = f.tile_y == d.tile_y && f.zchunk == d.zchunk && f.hold == d.hold ? c->box_default : 0;
+  c->box = 0;
   drop_graph(c);
+}
+
+extern "C" lbm_status lbm_set_box(lbm_ctx* c, int box) {
+  if (!c) return LBM_ERR_ARG;
+  if (box < 0 || box > 2) return fail(c, LBM_ERR_ARG, "box must be 0, 1 or 2");
+  if (box && (c->ncases > 1 || c->kernel != LBM_KERNEL_FUSED || c->cases[0].args.bgk))
+    return fail(c, LBM_ERR_ARG, "the box form steps single MRT lattices of the fused kernel");
+  if (box && (c->cases[0].p.ny > 4 * 65535 || c->cases[0].p.nz > 4 * 65535))
+    return fail(c, LBM_ERR_ARG, "the box form takes ny and nz up to 262140");
+  c->box = box;
+  drop_graph(c);
+  c->err[0] = 0;
+  return LBM_OK;
+}
+
+extern "C" int lbm_get_box(const lbm_ctx* c) { return c ? c->box : 0; }
+
+extern "C" lbm_status lbm_default_box(const lbm_params* p, int* box) {
+  g_create_err[0] = 0;
+  lbm_status st = validate_any_size(p);  // also of a lattice that only fits as slabs
+  if (st != LBM_OK) return st;
+  if (!box) return fail(nullptr, LBM_ERR_ARG, "lbm_default_box: NULL output");
+  *box = 0;
+  if (p->kernel == LBM_KERNEL_FUSED && (double)p->nx * p->ny * p->nz < 1e8) {
+    const long long N = (long long)p->nx * p->ny * p->nz;
+    *box = lbm::default_box(derive_args(p, (N + 63) / 64 * 64), p->storage);
+  }
+  return LBM_OK;
 }
 
 extern "C" lbm_status lbm_set_fused_config(lbm_ctx* c, int tile_y, int zchunk,

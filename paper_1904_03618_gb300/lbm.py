@@ -111,6 +111,12 @@ _lib.lbm_set_fused_config.argtypes = [_ctx_p, ctypes.c_int, ctypes.c_int, ctypes
 _lib.lbm_set_fused_config.restype = ctypes.c_int
 _lib.lbm_get_fused_config.argtypes = [_ctx_p] + [ctypes.POINTER(ctypes.c_int)] * 3
 _lib.lbm_get_fused_config.restype = ctypes.c_int
+_lib.lbm_set_box.argtypes = [_ctx_p, ctypes.c_int]
+_lib.lbm_set_box.restype = ctypes.c_int
+_lib.lbm_get_box.argtypes = [_ctx_p]
+_lib.lbm_get_box.restype = ctypes.c_int
+_lib.lbm_default_box.argtypes = [ctypes.POINTER(LbmParams), ctypes.POINTER(ctypes.c_int)]
+_lib.lbm_default_box.restype = ctypes.c_int
 _lib.lbm_create_batch.argtypes = [ctypes.POINTER(LbmParams), ctypes.c_int, ctypes.c_void_p,
                                   ctypes.POINTER(ctypes.c_void_p)]
 _lib.lbm_create_batch.restype = ctypes.c_int
@@ -183,6 +189,7 @@ EXPORTED = ("lbm_create", "lbm_init_fields", "lbm_step", "lbm_moments",
             "lbm_get_populations", "lbm_set_populations", "lbm_plane_bytes",
             "lbm_get_planes", "lbm_set_planes",
             "lbm_set_fused_config", "lbm_get_fused_config", "lbm_default_fused_config",
+            "lbm_set_box", "lbm_get_box", "lbm_default_box",
             "lbm_step_noalloc",
             "lbm_inplace_init", "lbm_inplace_set", "lbm_step_inplace", "lbm_inplace_read",
             "lbm_create_batch", "lbm_num_cases", "lbm_batch_init_fields",
@@ -390,6 +397,25 @@ def lbm_get_fused_config(ctx):
     v = [ctypes.c_int() for _ in range(3)]
     _check(ctx, _lib.lbm_get_fused_config(ctx, *[ctypes.byref(x) for x in v]))
     return tuple(x.value for x in v)
+
+
+def lbm_set_box(ctx, box):
+    """Steps of a single lattice in the box form (1: 4 x 4 x 4 cells per CTA,
+    2: 8 x 4 x 4) or the kernel of the fused configuration (0)."""
+    _check(ctx, _lib.lbm_set_box(ctx, int(box)))
+
+
+def lbm_get_box(ctx) -> int:
+    return _lib.lbm_get_box(ctx)
+
+
+def lbm_default_box(params: LbmParams) -> int:
+    """The box form lbm_create picks for this single lattice (host only)."""
+    v = ctypes.c_int()
+    st = _lib.lbm_default_box(ctypes.byref(params), ctypes.byref(v))
+    if st != LBM_OK:
+        raise LbmError(st, lbm_last_error(None))
+    return v.value
 
 
 def lbm_default_fused_config(params: LbmParams, sms=0):
