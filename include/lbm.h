@@ -254,7 +254,10 @@ lbm_status lbm_set_populations(lbm_ctx *ctx, const void *src);
    state within two planes, so after every step the two outermost planes
    of each neighbour's own range, copied into the ghost planes, make the
    slab's own planes evolve exactly as in the undivided lattice (the ghost
-   planes themselves are overwritten by the next copy).
+   planes themselves are overwritten by the next copy) -- where both run the
+   same form of the step, which depends on x and y alone except for the box
+   form of small lattices: give a slab's context the undivided lattice's,
+   lbm_set_box(slab, box) with box from lbm_default_box.
    lbm_get_planes copies the stored planes z0 .. z0 + n - 1 of the current
    state into dst, lbm_set_planes copies src into them: raw storage format
    (the buffer the next step pulls from; FP16 / BF16 as stored

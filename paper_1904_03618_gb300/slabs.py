@@ -126,6 +126,13 @@ class SlabPlan:
         return out
 
 
+def whole_box(pd: dict, storage: str) -> int:
+    """The box form (lbm_default_box) of the undivided lattice: its slabs run
+    it too, smaller than it though they are, so that they step exactly as it."""
+    from . import lbm
+    return lbm.lbm_default_box(lbm.make_params(storage=storage, **pd))
+
+
 def split_fields(plan: SlabPlan, fields):
     """The slab's local initial fields (own planes plus ghosts, periodic in
     z where the lattice is) from the whole lattice's (rho_R, rho_B, u) in
@@ -189,6 +196,7 @@ class SlabLattice:
         self.params.ref_R, self.params.ref_B = refs
         self.stream = torch.cuda.current_stream(self.device)
         self.lat = lbm.Lattice(self.params, device=self.device, stream=self.stream)
+        lbm.lbm_set_box(self.lat.ctx, whole_box(pd, storage))
         nbytes = lbm.lbm_plane_bytes(self.lat.ctx)
         self.plane_words = nbytes // 4   # exchanged as 32-bit words
         self._buf = {}
@@ -252,6 +260,7 @@ class SlabsOnOneDevice:
             p = lbm.make_params(storage=storage, **plan.local_params(pd))
             p.ref_R, p.ref_B = refs
             self.lats.append(lbm.Lattice(p, device=self.device, stream=self.stream))
+            lbm.lbm_set_box(self.lats[-1].ctx, whole_box(pd, storage))
         self.plane_bytes = lbm.lbm_plane_bytes(self.lats[0].ctx)
         self._tmp = torch.empty(GHOST * self.plane_bytes // 4, dtype=torch.int32,
                                 device=self.device)
