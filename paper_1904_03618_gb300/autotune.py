@@ -2,13 +2,14 @@
 
 The fused kernel's launch configuration -- tile height, planes per CTA
 (z chunk) and where a plane's reduced state waits between its pull and its
-collision -- does not change results (the parity tests run every
-configuration against the oracle); it only changes speed, and the best
-choice depends on the lattice shape, the storage type and, for batches, on
-the mix of box sizes.  `tune` times the candidate configurations on the
-live context with CUDA events on its stream, keeps the fastest, applies it,
-and records it in a JSON cache keyed by device, storage and lattice
-signature so that later runs of the same shape skip the timing.
+collision -- changes results by rounding only (the parity tests run every
+configuration against the oracle), and the best choice depends on the
+lattice shape, the storage type and, for batches, on the mix of box sizes.
+`tune` times the candidate configurations on the live context with CUDA
+events on its stream, among them what lbm_create picks (on small lattices
+the box form), keeps the fastest, applies it, and records it in a JSON cache
+keyed by device, storage, collision operator and lattice signature so that
+later runs of the same shape skip the timing.
 
 Timing advances the context's state (it runs real steps).  Tune before
 initialising the run that matters, or accept the extra steps.
@@ -35,6 +36,10 @@ DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "paper_1904_0361
                              "autotune.json")
 
 
+# of the library's set of forms: entries timed among other forms do not apply
+FORMS = 2
+
+
 def signature(params_list, storage: int) -> str:
     """Cache key of a lattice (one params) or a batch (several)."""
     dev = torch.cuda.get_device_name()
@@ -47,7 +52,8 @@ def signature(params_list, storage: int) -> str:
         for s in sizes:
             counts[s] = counts.get(s, 0) + 1
         shape = "batch:" + ",".join("%dx%dx%d*%d" % (k + (v,)) for k, v in sorted(counts.items()))
-    return "%s|storage%d|%s" % (dev, storage, shape)
+    return "%s|storage%d|%s|collision%d|forms%d" % (dev, storage, shape, params_list[0].collision,
+                                                    FORMS)
 
 
 def _load(path):
@@ -66,10 +72,20 @@ def _store(path, table):
     os.replace(tmp, path)
 
 
+def _apply(ctx, tile_y, zchunk, hold, box):
+    """The configuration, or with box > 0 the box form beside it."""
+    lbm.lbm_set_fused_config(ctx, tile_y, zchunk, hold)
+    if box:
+        lbm.lbm_set_box(ctx, box)
+
+
 def _time(ctx, stream, steps):
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
-    lbm.lbm_step(ctx, 2)  # warm-up (and graph capture for this configuration)
+    warmup = 4  # captures the graph that the timed steps replay
+    if lbm.lbm_get_box(ctx):
+        warmup, steps = 20, max(steps, 32)  # 16 steps to a graph
+    lbm.lbm_step(ctx, warmup)
     e0.record(stream)
     lbm.lbm_step(ctx, steps)
     e1.record(stream)
@@ -82,36 +98,42 @@ def tune(ctx, params_list, stream, steps=8, cache_path=DEFAULT_CACHE, use_cache=
     """Chooses and applies the fastest fused configuration for `ctx` (a
     Lattice's or Batch's context; every case must be initialised).  Returns
     (tile_y, zchunk, hold, ms_per_step, source) with source "cache" or
-    "timed"."""
+    "timed"; whether the box form steps beside it, lbm_get_box tells."""
     params_list = list(params_list)
     storage = int(params_list[0].storage)
     key = signature(params_list, storage)
     table = _load(cache_path) if (use_cache and cache_path) else {}
     if use_cache and key in table:
         t = table[key]
-        lbm.lbm_set_fused_config(ctx, t["tile_y"], t["zchunk"], t["hold"])
-        return t["tile_y"], t["zchunk"], t["hold"], t["ms"], "cache"
+        try:
+            _apply(ctx, t["tile_y"], t["zchunk"], t["hold"], t["box"])
+            return t["tile_y"], t["zchunk"], t["hold"], t["ms"], "cache"
+        except (KeyError, lbm.LbmError):
+            pass  # not of this context after all: time it
     if candidates is None:
         shapes = BATCH_SHAPES if len(params_list) > 1 else SINGLE_SHAPES
         nz = max(p.nz for p in params_list)
         candidates = [(ty, zc, hold) for ty, hold in shapes for zc in ZCHUNKS if zc <= max(nz, 8)]
-        if len(params_list) == 1:  # the context's own choice (small lattices: the box form)
-            candidates.insert(0, lbm.lbm_get_fused_config(ctx))
+        if len(params_list) == 1:  # what lbm_create picks, whatever the context runs now
+            sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+            p = params_list[0]
+            candidates.insert(0, lbm.lbm_default_fused_config(p, sms) + (lbm.lbm_default_box(p),))
     best = None
-    for ty, zc, hold in candidates:
+    for ty, zc, hold, box in (tuple(c) + (0,) * (4 - len(c)) for c in candidates):
         try:
-            lbm.lbm_set_fused_config(ctx, ty, zc, hold)
+            _apply(ctx, ty, zc, hold, box)
         except lbm.LbmError:
             continue
         ms = _time(ctx, stream, steps)
-        if best is None or ms < best[3]:
-            best = (ty, zc, hold, ms)
+        if best is None or ms < best[4]:
+            best = (ty, zc, hold, box, ms)
     if best is None:
         raise RuntimeError("autotune: no valid configuration")
-    lbm.lbm_set_fused_config(ctx, best[0], best[1], best[2])
+    ty, zc, hold, box, ms = best
+    _apply(ctx, ty, zc, hold, box)
     if cache_path:
         table = _load(cache_path)
-        table[key] = {"tile_y": best[0], "zchunk": best[1], "hold": best[2], "ms": best[3],
+        table[key] = {"tile_y": ty, "zchunk": zc, "hold": hold, "box": box, "ms": ms,
                       "when": time.strftime("%Y-%m-%dT%H:%M:%S")}
         _store(cache_path, table)
-    return best + ("timed",)
+    return ty, zc, hold, ms, "timed"
