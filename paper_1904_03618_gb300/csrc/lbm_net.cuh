@@ -408,10 +408,15 @@ __global__ void __launch_bounds__(kNetThreads, 1)
                 store4(yp, c + 4, N, vec, v + 4);
               }
             } else {
-              // columns from N to its padding are k of the next product: zero
-              // (bias and weights are zero there, tanh(0) = 0)
 #pragma unroll
               for (int i = 0; i < 8; ++i) v[i] = net_tanh(v[i]);
+              // columns from N to its padding are k of the next product: zero, also
+              // where an infinite input has made a NaN of their zero weights
+              if (c + 8 > N) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                  if (c + i >= N) v[i] = 0.f;
+              }
               *reinterpret_cast<uint4*>(act + act_offset(row, c)) = pack8(v);
             }
           }
