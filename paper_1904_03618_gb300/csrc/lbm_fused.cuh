@@ -36,13 +36,12 @@ namespace lbm {
 
 constexpr int kTileW = 32;  // threads along x per CTA (one warp)
 
-// Both colours in one paired add (two roundings as of two adds).  GB300, us: 192
-// x 192 x 768 BF16 12,430 -> 12,360 per 8 steps, FP16 droplet sweep 14,285 ->
-// 14,150 per 12, 128^3 FP16 3629 -> 3662 per 30.
 template <typename T, int I>
 __device__ __forceinline__ void add_offsets(const StepArgs& a, float2& v) {
-  if (Store<T>::kDeviation)
-    v = __fadd2_rn(v, make_float2(dev_offset<I>(a, 0), dev_offset<I>(a, 1)));
+  if (Store<T>::kDeviation) {
+    v.x += dev_offset<I>(a, 0);
+    v.y += dev_offset<I>(a, 1);
+  }
 }
 
 // Pull of the 19 pairs of one column / plane, reduced on the fly to
