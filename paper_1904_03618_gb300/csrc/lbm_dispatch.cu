@@ -360,8 +360,11 @@ class BatchSpan {
 // 96 cells 1268 / 1535 / 1481; 16 bits, 34 x 15 / 32 x 8: 60 of 40 x 40 x 24 326 /
 // 241, 60 of 64 x 72 x 32 670 / 812.  The seam form only where no box is narrower
 // than its tile (the droplet boxes' 32-cell ones are what slows it there).  A
-// batch of fewer than 32 CTAs keeps the tensor-copy form, whose bounded waits
-// the fault tests step.
+// batch of fewer than 32 CTAs keeps the tensor-copy form, the slower one there
+// (three boxes of 40 x 40 x 24 100 us against 31 on the 32 x 8 tile, two of 32^3
+// and two of 64 x 64 x 32 133 and 131 against 31 and 42): its bounded waits and
+// their report are what is specified of the smallest batches; lbm_set_fused_config
+// gives a program the faster form.
 void batch_default_config(const StepArgs* const* args, int ncases, int storage, int sms,
                           bool seam_ok, FusedConfig* c) {
   BatchSpan t15(sms), t12(sms), t8(2 * sms);
@@ -419,14 +422,17 @@ FusedConfig default_fused_config(const StepArgs& a, int storage) {
   return c;
 }
 
-// The box form's range, GB300, us per step (box / the fastest marching chunk):
-// with walls 45^3 11.3 / 16.5, 59^3 21.3 / 20.6, 60^3 20.7 / 18.5; FP16 45^3 9.6 /
-// 13.3, 59^3 18.7 / 17.4; BGK 45^3 10.3 / 14.3, 59^3 20.0 / 17.4, 120 x 70 x 29
-// FP16 21.3 / 18.9; 101 x 50 x 50 25.3 / 20.5: it wins up to about 180,000 cells.
-// On the lattices of the seam forms, the line lies lower than that, at 81,920
-// cells: from there on the tensor-copy kernel with its bounded waits, which
-// reports them in the error word, is the documented default (the fault tests
-// step a 64 x 40 x 36 lattice through it).
+// The box form's range, GB300, us per step (box / the fastest marching chunk).
+// Without a seam form it wins up to about 180,000 cells: walls all round 45^3
+// 11.4 / 14.4, 53^3 17.0 / 18.4, 57^3 21.2 / 18.4, 59^3 21.4 / 18.4; FP16 10.5 /
+// 14.3, 15.9 / 17.4, 19.3 / 17.4, 19.5 / 17.4.
+// On the lattices of the seam forms the line at 81,920 cells is not where the two
+// are equal: 64 x 40 x 32 9.2 / 24.6, 64 x 40 x 36 (beyond it) 9.5 / 25.6, 48^3 10.6
+// / 24.6, 56^3 16.2 / 24.7, 64^3 23.9 / 28.5, 72^3 36.2 / 39.9; FP16 48^3 9.7 / 13.3,
+// 56^3 14.9 / 16.4, 60^3 18.8 / 16.4, 64^3 21.7 / 28.7.  It keeps the tensor-copy
+// kernels, whose bounded waits report through the error word, the default of the
+// lattices on which that is specified (from 92,160 cells on); lbm_set_box gives a
+// program the faster form there.
 // BGK lattices keep the shared-memory-hold kernel: its multiply-adds and the box
 // form's are contracted differently, and under that operator a changed last bit
 // grows near tau_v = 1/2 (a closed box of drops 4e-5 apart after 60 steps, a

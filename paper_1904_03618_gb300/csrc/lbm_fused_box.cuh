@@ -12,13 +12,15 @@
 // barrier and one collision, spread over every SM.  The ring's pulls are
 // redundant (a 4 x 4 x 4 box pulls 208 cells for 64, an 8 x 4 x 4 box 352 for
 // 128) but hit L2, which holds both buffers at these sizes.  GB300, us per
-// step in a run of 400, marching kernel -> box: 4 x 128 x 4 with walls 19.5
-// -> 2.5, 16^3 17.4 -> 3.1, 24^3 18.3 -> 3.6, 32^3 26.7 -> 4.4, 40^3 24.6 ->
-// 7.3, 48 x 48 x 32 FP16 13.3 -> 6.8.  Which box: 4 x 4 x 4 while its CTAs
-// leave SMs idle or nearly so (24^3: 216 CTAs 3.6, 8 x 4 x 4 3.9), the larger
-// box with less ring from there on (32^3: 512 CTAs 6.4, 256 CTAs 4.4); 8 x 8
-// x 4 and 16 x 4 x 4 boxes were no faster anywhere (32^3 4.5 and 4.3, 48^3
-// 12.0 and 11.5 against 10.8).
+// step in a run of 200, marching kernel -> box: 4 x 128 x 4 with walls 19.6
+// -> 2.6, 16^3 16.4 -> 2.7, 24^3 17.6 -> 3.5, 32^3 26.4 -> 4.4, 40^3 24.6 ->
+// 7.2, FP16 13.3 -> 6.7.  Which box: 4 x 4 x 4 while its CTAs leave SMs idle
+// (20^3: 125 CTAs 2.7, 8 x 4 x 4 3.1), the larger box with less ring on more
+// cells (32^3: 512 CTAs 6.8, 256 CTAs 4.4).  The two are level at about 10,000
+// cells (22^3 3.4 / 3.2, 25^3 4.2 / 4.4, 32 x 32 x 16 4.7 / 3.2); the line in
+// default_box, 16,384, is that of an earlier overlap of the launches, under
+// which 24^3 took 3.6 / 3.9.  8 x 8 x 4 and 16 x 4 x 4 boxes were no faster
+// anywhere (then: 32^3 4.5 and 4.3, 48^3 12.0 and 11.5 against 10.8).
 #pragma once
 
 #include "lbm_fused.cuh"

@@ -114,7 +114,7 @@ cudaError_t launch_fused(int storage, const void* src, void* dst,
 FusedConfig default_fused_config(const StepArgs& a, int storage);
 // Box form of the step for small lattices (lbm_fused_box.cuh): box 1 = 4 x 4
 // x 4 cells per CTA, 2 = 8 x 4 x 4; default_box 0: the lattice is large
-// enough for the marching kernels.
+// enough for the marching kernels, or BGK.
 int default_box(const StepArgs& a, int storage);
 template <typename T>
 cudaError_t launch_fused_box_storage(const void* src, void* dst, const StepArgs& a, int box,
