@@ -71,3 +71,28 @@ def test_in_place_step_rounds_alike(column):
         assert abs(_rms(lat.get_f(), ref) / base - 1) <= 0.01
     finally:
         lat.close()
+
+
+def test_a_case_of_a_batch_steps_as_the_lattice_alone(column):
+    """To the contraction of multiply-add pairs: a few ulp of the largest
+    population per step, 1e-6 of it after three."""
+    pd, f0, _ = column
+    p = lbm.make_params(**pd)
+    alone = lbm.Lattice(p, device=DEV)
+    try:
+        alone.set_f(f0)
+        alone.step(3)
+        want = alone.get_f()
+    finally:
+        alone.close()
+    for config in [(8, 9, 2)] + ([(12, 0, 7), (15, 0, 8)] if pd["collision"] == "mrt" else []):
+        b = lbm.Batch([p, p], device=DEV)
+        try:
+            lbm.lbm_set_fused_config(b.ctx, *config)
+            for k in (0, 1):
+                b.set_f(k, f0)
+            b.step(3)
+            for k in (0, 1):
+                assert (b.get_f(k) - want).abs().max() <= 1e-6 * want.abs().max(), (config, k)
+        finally:
+            b.close()
